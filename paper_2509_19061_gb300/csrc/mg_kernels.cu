@@ -159,73 +159,197 @@ __global__ void k_assemble(const DenseJob *__restrict__ jobs)
     A[(size_t)r * n + c] = -m;
 }
 
-// In-place Cholesky A = L L^T (lower triangle) by one CTA per job
-// (blockIdx.x); status = 1 if a pivot is not positive.  Every entry is
-// updated in the order k = 0, 1, ..., whatever the thread layout.
-__global__ void k_cholesky(const DenseJob *__restrict__ jobs)
-{
-    const DenseJob &jb = jobs[blockIdx.x];
-    const int n = jb.n;
-    double *__restrict__ A = jb.A;
-    __shared__ double piv;
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            const double d = A[(size_t)k * n + k];
-            if (!(d > 0.0)) bad = 1;
-            piv = d > 0.0 ? sqrt(d) : 1.0;
-            A[(size_t)k * n + k] = piv;
-        }
-        __syncthreads();
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) A[(size_t)i * n + k] /= piv;
-        __syncthreads();
-        // trailing lower triangle, rows/cols k+1..n-1: warp w takes rows
-        // k+1+w, k+1+w+nw, ..., its lanes the columns of a row
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        for (int i = k + 1 + w; i < n; i += nw) {
-            const double lik = A[(size_t)i * n + k];
-            for (int j = k + 1 + lane; j <= i; j += 32) A[(size_t)i * n + j] -= lik * A[(size_t)j * n + k];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && bad) *jb.status = 1;
-}
+// The dense factorisation -M = L L^T, W = L^{-1}, (-M)^{-1} = W^T W of one
+// coarsest level (n <= 1024) is bound by the FP64 pipe's latency and rate (two
+// FP64 lanes per clock and SM) and by its chain of n square roots and
+// divisions, not by bytes (n^2 doubles stay in L2).  One CTA per matrix kept
+// one SM's FP64 pipe for the whole n^3 / 6: 12.4 ms for L and 12.5 ms for W at
+// n = 480.  Blocked by 32 columns the work spreads over the SMs and only the
+// chain stays serial: 0.86 and 0.43 ms (and 0.065 for W^T W, from 0.157).  Every entry is still formed by the same operations in
+// the same order (its updates in ascending k, then its division), so the
+// factors have the bits of the unblocked algorithm.
+constexpr int DN_B = 32;  // block columns
+constexpr int DN_ER = 16; // rows below the diagonal block per panel CTA
 
-// W = L^{-1}, column c by thread c (forward substitution), lower triangle;
-// one job per blockIdx.y
-__global__ void k_tri_inverse(const DenseJob *__restrict__ jobs)
+// Panel kb: the diagonal block's factor (formed by every CTA, from the
+// trailing matrix in A) and DN_ER rows of the block column below it, into the
+// lower triangle of `L` (the job's Ainv buffer, free until k_gram).  The
+// diagonal block and the CTA's rows go through the columns together.  `status`
+// is set to 1 if a pivot is not positive.  Grid: (row groups, jobs).
+__global__ void __launch_bounds__(256) k_chol_panel(const DenseJob *__restrict__ jobs, int kb)
 {
     const DenseJob &jb = jobs[blockIdx.y];
-    const int n = jb.n;
-    const double *__restrict__ L = jb.A;
+    const int n = jb.n, k0 = kb * DN_B;
+    if (k0 >= n) return;
+    const int r0 = k0 + DN_B + (int)blockIdx.x * DN_ER; // first row of this CTA below the block
+    if (blockIdx.x > 0 && r0 >= n) return;
+    const double *__restrict__ A = jb.A;
+    double *__restrict__ L = jb.Ainv;
+    constexpr int ROWS = DN_B + DN_ER;
+    __shared__ double P[ROWS][DN_B + 1]; // rows 0..31: the diagonal block
+    const int nb = min(DN_B, n - k0), tid = (int)threadIdx.x;
+    auto row_of = [&](int q) { return q < DN_B ? k0 + q : r0 + (q - DN_B); };
+    for (int e = tid; e < ROWS * DN_B; e += 256) {
+        const int q = e / DN_B, c = e % DN_B, i = row_of(q);
+        P[q][c] = (i < n && c < nb && (q >= DN_B || c <= q)) ? A[(size_t)i * n + k0 + c] : 0.0;
+    }
+    bool bad = false;
+    const int rows = r0 < n ? DN_B + min(DN_ER, n - r0) : DN_B;
+    for (int k = 0; k < nb; ++k) {
+        __syncthreads();
+        const double d = P[k][k];
+        if (!(d > 0.0)) bad = true;
+        double v = 0.0;
+        if (tid < rows && tid >= k) { // one thread per row of the column
+            const double piv = d > 0.0 ? sqrt(d) : 1.0;
+            v = tid == k ? piv : P[tid][k] / piv;
+        }
+        __syncthreads();
+        if (tid < rows && tid >= k) P[tid][k] = v;
+        __syncthreads();
+        // columns k + 1 .. of every row below k: warp w takes columns k + 1 + w, ...
+        const int lane = tid & 31, w = tid >> 5;
+        for (int c = k + 1 + w; c < nb; c += 8) {
+            const double lc = P[c][k];
+            if (lane >= c) P[lane][c] = fma(-P[lane][k], lc, P[lane][c]);
+            if (lane < DN_ER) P[DN_B + lane][c] = fma(-P[DN_B + lane][k], lc, P[DN_B + lane][c]);
+        }
+    }
+    __syncthreads();
+    const int q0 = blockIdx.x == 0 ? 0 : DN_B;
+    for (int e = tid + q0 * DN_B; e < rows * DN_B; e += 256) {
+        const int q = e / DN_B, c = e % DN_B, i = row_of(q);
+        if (i < n && c < nb && (q >= DN_B || c <= q)) L[(size_t)i * n + k0 + c] = P[q][c];
+    }
+    if (bad && tid == 0 && blockIdx.x == 0) *jb.status = 1;
+}
+
+// Trailing update of panel kb: A[i][j] -= sum_k L[i][k] L[j][k] over the
+// panel's columns in ascending k, one 16 x 16 tile of the lower triangle per
+// CTA (one entry per thread; 16 x 16 keeps all SMs busy until the trailing
+// matrix is small).  Grid: (tiles of the largest trailing triangle, jobs).
+__global__ void __launch_bounds__(256) k_chol_update(const DenseJob *__restrict__ jobs, int kb)
+{
+    const DenseJob &jb = jobs[blockIdx.y];
+    const int n = jb.n, k0 = kb * DN_B, t0 = k0 + DN_B;
+    if (t0 >= n) return;
+    const double *__restrict__ L = jb.Ainv;
+    double *__restrict__ A = jb.A;
+    // tile (I, J), J <= I, of the lower triangle numbered row by row
+    const int b = (int)blockIdx.x;
+    int I = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
+    while ((I + 1) * (I + 2) / 2 <= b) ++I;
+    while (I * (I + 1) / 2 > b) --I;
+    const int J = b - I * (I + 1) / 2;
+    const int i0 = t0 + 16 * I, j0 = t0 + 16 * J;
+    if (i0 >= n) return;
+    __shared__ double Li[16][DN_B + 1], Lj[16][DN_B + 1];
+    const int tid = (int)threadIdx.x;
+    for (int e = tid; e < 16 * DN_B; e += 256) {
+        const int q = e / DN_B, c = e % DN_B;
+        Li[q][c] = i0 + q < n ? L[(size_t)(i0 + q) * n + k0 + c] : 0.0;
+        Lj[q][c] = j0 + q < n ? L[(size_t)(j0 + q) * n + k0 + c] : 0.0;
+    }
+    __syncthreads();
+    const int i = i0 + tid / 16, j = j0 + tid % 16;
+    if (i >= n || j > i) return;
+    double a = A[(size_t)i * n + j];
+#pragma unroll 8
+    for (int c = 0; c < DN_B; ++c) a = fma(-Li[tid / 16][c], Lj[tid % 16][c], a);
+    A[(size_t)i * n + j] = a;
+}
+
+// W = L^{-1} (lower triangle; zero above), C columns per CTA, one thread per
+// (row of the current 32-row block, column): the block's sums over the rows
+// above it from 32 x 32 tiles of L (ascending m), then the block's forward
+// substitution.  The columns' finished part stays in shared memory.  C = 4
+// spreads one matrix over n / 4 CTAs (chain-bound); C = 16 uses the lanes of
+// the divisions better and is for many matrices at once (FP64-rate-bound).
+// Grid: (column groups, jobs); dynamic shared memory n_max x C doubles.
+template <int C>
+__global__ void __launch_bounds__(DN_B *C) k_tri_inverse(const DenseJob *__restrict__ jobs)
+{
+    extern __shared__ __align__(16) double Wc[]; // [row][C]
+    const DenseJob &jb = jobs[blockIdx.y];
+    const int n = jb.n, c0 = (int)blockIdx.x * C;
+    if (c0 >= n) return;
+    const double *__restrict__ L = jb.Ainv;
     double *__restrict__ W = jb.W;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    for (int i = 0; i < c; ++i) W[(size_t)i * n + c] = 0.0;
-    W[(size_t)c * n + c] = 1.0 / L[(size_t)c * n + c];
-    for (int i = c + 1; i < n; ++i) {
+    __shared__ double T[DN_B][DN_B + 1];
+    const int tid = (int)threadIdx.x, r = tid / C, q = tid % C, c = c0 + q;
+    const int b0 = c0 / DN_B, nblk = (n + DN_B - 1) / DN_B;
+    auto load_tile = [&](int I, int K) { // rows of block I, columns of block K, zero outside the triangle
+        for (int e = tid; e < DN_B * DN_B; e += DN_B * C) {
+            const int i = I * DN_B + e / DN_B, m = K * DN_B + e % DN_B;
+            T[e / DN_B][e % DN_B] = (i < n && m <= i) ? L[(size_t)i * n + m] : 0.0;
+        }
+    };
+    if (c < n)
+        for (int i = r; i < b0 * DN_B; i += DN_B) W[(size_t)i * n + c] = 0.0;
+    for (int I = b0; I < nblk; ++I) {
         double s = 0.0;
-        for (int m = c; m < i; ++m) s += L[(size_t)i * n + m] * W[(size_t)m * n + c];
-        W[(size_t)i * n + c] = -s / L[(size_t)i * n + i];
+        for (int K = b0; K < I; ++K) {
+            __syncthreads();
+            load_tile(I, K);
+            __syncthreads();
+            const double *wk = Wc + (size_t)K * DN_B * C + q;
+#pragma unroll 4
+            for (int m = 0; m < DN_B; ++m) s = fma(T[r][m], wk[m * C], s);
+        }
+        __syncthreads();
+        load_tile(I, I);
+        __syncthreads();
+        const int i0 = I * DN_B, nr = min(DN_B, n - i0);
+        for (int t = 0; t < nr; ++t) {
+            if (r == t) {
+                const int i = i0 + t;
+                double w = 0.0;
+                if (c < n && i == c) w = 1.0 / T[t][t];
+                else if (c < n && i > c) w = -s / T[t][t];
+                Wc[(size_t)i * C + q] = w;
+                if (c < n) W[(size_t)i * n + c] = w;
+            }
+            __syncthreads();
+            if (r > t && i0 + t >= c) s = fma(T[r][t], Wc[(size_t)(i0 + t) * C + q], s);
+        }
     }
 }
 
-// Ainv = W^T W; one job per blockIdx.y
-__global__ void k_gram(const DenseJob *__restrict__ jobs)
+// Ainv = W^T W, one 16 x 16 tile of the lower triangle per CTA (an entry per
+// thread, ascending m from the tile's first row) stored to both triangles
+// (the products commute, so the mirrored entry has the same bits).  Grid:
+// (tiles of the largest triangle, jobs).
+__global__ void __launch_bounds__(256) k_gram(const DenseJob *__restrict__ jobs)
 {
     const DenseJob &jb = jobs[blockIdx.y];
     const int n = jb.n;
     const double *__restrict__ W = jb.W;
     double *__restrict__ Ainv = jb.Ainv;
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)n * n) return;
-    const int i = (int)(t / n), j = (int)(t - (long)i * n);
-    const int m0 = i > j ? i : j;
+    const int b = (int)blockIdx.x;
+    int I = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
+    while ((I + 1) * (I + 2) / 2 <= b) ++I;
+    while (I * (I + 1) / 2 > b) --I;
+    const int J = b - I * (I + 1) / 2;
+    const int i0 = 16 * I, j0 = 16 * J;
+    if (i0 >= n) return;
+    __shared__ double Wi[DN_B][16], Wj[DN_B][16];
+    const int tid = (int)threadIdx.x, ti = tid / 16, tj = tid % 16;
     double s = 0.0;
-    for (int m = m0; m < n; ++m) s += W[(size_t)m * n + i] * W[(size_t)m * n + j];
+    for (int m0 = i0; m0 < n; m0 += DN_B) { // W[m][i] = 0 for m < i, and j <= i
+        __syncthreads();
+        for (int e = tid; e < DN_B * 16; e += 256) {
+            const int m = m0 + e / 16, q = e % 16;
+            Wi[e / 16][q] = (m < n && i0 + q < n) ? W[(size_t)m * n + i0 + q] : 0.0;
+            Wj[e / 16][q] = (m < n && j0 + q < n) ? W[(size_t)m * n + j0 + q] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int m = 0; m < DN_B; ++m) s = fma(Wi[m][ti], Wj[m][tj], s);
+    }
+    const int i = i0 + ti, j = j0 + tj;
+    if (i >= n || j > i) return;
     Ainv[(size_t)i * n + j] = s;
+    Ainv[(size_t)j * n + i] = s;
 }
 
 // pack the coarsest right-hand side into a dense FP64 vector
@@ -315,13 +439,30 @@ template <typename T>
 cudaError_t mg_dense_setup_many(const DenseJob *jobs, int count, int nmax, cudaStream_t s)
 {
     const long nn = (long)nmax * nmax;
+    const int nblk = (nmax + DN_B - 1) / DN_B;
+    auto tiles16 = [](int rows) { const int t = (rows + 15) / 16; return (unsigned)(t * (t + 1) / 2); };
+    // four columns per CTA while that leaves at most four CTAs an SM (480
+    // unknowns: 120 CTAs a matrix), where the chain bounds it; sixteen beyond,
+    // where the FP64 rate does and a division wants full warps
+    const bool many = (long)count * ((nmax + 3) / 4) > 4L * 152;
+    const int cols = many ? 16 : 4;
+    const size_t wsm = (size_t)nblk * DN_B * cols * sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(many ? k_tri_inverse<16> : k_tri_inverse<4>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm);
+    if (e != cudaSuccess) return e;
     for (int j0 = 0; j0 < count; j0 += 65535) {
         const int c = count - j0 < 65535 ? count - j0 : 65535;
         const DenseJob *jb = jobs + j0;
         k_assemble<T><<<dim3((unsigned)((nn + 255) / 256), c), 256, 0, s>>>(jb);
-        k_cholesky<<<c, 1024, 0, s>>>(jb);
-        k_tri_inverse<<<dim3((nmax + 127) / 128, c), 128, 0, s>>>(jb);
-        k_gram<<<dim3((unsigned)((nn + 255) / 256), c), 256, 0, s>>>(jb);
+        for (int kb = 0; kb < nblk; ++kb) {
+            const int below = nmax - (kb + 1) * DN_B; // rows below the diagonal block
+            k_chol_panel<<<dim3((unsigned)(below > 0 ? (below + DN_ER - 1) / DN_ER : 1), c), 256, 0, s>>>(jb, kb);
+            if (below > 0) k_chol_update<<<dim3(tiles16(below), c), 256, 0, s>>>(jb, kb);
+        }
+        const dim3 gi((unsigned)((nmax + cols - 1) / cols), c);
+        if (many) k_tri_inverse<16><<<gi, DN_B * 16, wsm, s>>>(jb);
+        else k_tri_inverse<4><<<gi, DN_B * 4, wsm, s>>>(jb);
+        k_gram<<<dim3(tiles16(nmax), c), 256, 0, s>>>(jb);
     }
     return cudaGetLastError();
 }

@@ -126,6 +126,19 @@ def test_single_level_is_the_dense_solve(api):
     assert rel(v, (dx, dy)) <= 1e-11
 
 
+@pytest.mark.parametrize("nx,ny", [(2, 2), (5, 4), (3, 7), (4, 5), (2, 22), (7, 5), (9, 8), (16, 16), (20, 24),
+                                   (2, 342)])
+def test_dense_factorisation_sizes(api, nx, ny):
+    """The blocked dense solve at 4, 31, 32, 31, 64, 58, 127, 480, 916 and 1024
+    (the largest) unknowns, around the 32-column blocks.  Square cells; the
+    bound is that of the 16 x 12 solve above scaled by the growth of the
+    condition number, (side / 16)^2."""
+    prob = inputs.sinker_problem(nx, ny, eta_in=10.0, radius=0.3, ly=ny / nx)
+    st, e, c, v = run_solve(api, prob, "f64", 1, inner="f64", levels=1, variant="fused")
+    ref = ora.dense_solve(ogrid(prob), prob.fx, prob.fy)
+    assert rel(v, ref) <= 1e-11 * max(1.0, (max(nx, ny) / 16.0) ** 2)
+
+
 @pytest.mark.parametrize("inner", ["f64", "f32"])
 def test_solve_to_1e8_fp32_inner_reaches_the_fp64_solution(api, inner):
     """Flexible CG in FP64 around the V-cycle reaches E_v <= 1e-8 on the
