@@ -49,6 +49,7 @@ FLOPS_PER_CELL_SWEEP = 24
 NOMINAL_FP32_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 NOMINAL_FP64_TFLOPS = 1.25
 RAS_SOURCES = ["paper_2509_19061_gb300/csrc/ras_kernels.cu", "paper_2509_19061_gb300/csrc/stencil.cuh"]
+STREAM_SOURCES = ["paper_2509_19061_gb300/csrc/stream_kernels.cu", "paper_2509_19061_gb300/csrc/f32x2.cuh"]
 
 
 def parse():
@@ -321,8 +322,11 @@ def workload_config(args):
 TILE_KERNEL_NAMES = {"pair": "k_ras_pair", "tma": "k_ras_tma", "global": "k_ras_reg", "shared": "k_ras"}
 
 
-def tile_kernel_name(api, n, tile, overlap, dt_name):
-    """Name of the tile kernel the library picks for this launch shape."""
+def tile_kernel_name(api, n, tile, k, overlap, dt_name):
+    """Name of the kernel the library picks for this schedule: row streaming
+    where it equals global Jacobi on a large FP32 grid, else a tile kernel."""
+    if dt_name == "f32" and overlap >= k - 1 and n * n >= 600000:
+        return "k_ras_stream"
     return TILE_KERNEL_NAMES[api.stokes_tile_kernel_plan(n, n, tuple(tile), overlap, dt_name)[0]]
 
 
@@ -419,30 +423,33 @@ def run_ours(args):
 
     # roofline of the dominant kernel (the RAS tile kernel).  One launch runs
     # sweeps_per_launch local sweeps over every cell (the last launch of a step
-    # runs the remainder).  Its bound is the FP32 (FP64) pipe, not HBM (ncu:
-    # issue- and FMA-pipe-bound, DRAM well below peak), so the roofline is the
-    # arithmetic one: algorithmic flops of the owned cells per launch over the
-    # nominal arithmetic peak.  The HBM view is reported beside it twice: the
+    # runs the remainder).  The row-streaming kernel is bound by HBM.  A tile
+    # kernel's bound is the FP32 (FP64) pipe, not HBM (ncu: issue- and
+    # FMA-pipe-bound, DRAM well below peak), so its roofline is the arithmetic
+    # one: algorithmic flops of the owned cells per launch over the nominal
+    # arithmetic peak.  The HBM view is reported beside it twice: the
     # launch's minimum DRAM bytes (each field read once, vx and vy written
     # once: 8 words per cell per launch), and the effective bytes of the
     # paper's yardstick (8 words per cell per sweep, which exceeds the HBM
     # peak when k > 1 because the window stays on chip for k sweeps).
-    sweeps_per_launch = args.sweeps / math.ceil(args.sweeps / k)
+    kernel = tile_kernel_name(api, n, args.tile, k, o, dt_name)
+    sweeps_per_launch = args.sweeps * args.steps / max(ras_groups, 1)
     min_bytes = WORDS_PER_CELL_SWEEP * esize * cells
     eff_bytes = min_bytes * sweeps_per_launch
     avg_ms = ras_ms / max(ras_groups, 1)
     avg_s = avg_ms / 1e3
     peak, peak_kind = measured_peaks()
     key = "ras_%s_%d_t%dx%d_k%d_o%d" % (dt_name, n, args.tile[0], args.tile[1], k, o)
-    traffic = ncu_traffic(key, source_hash(RAS_SOURCES))
-    limiter = (ncu_entry(key, source_hash(RAS_SOURCES)) or {}).get("limiter")
+    sources = source_hash(STREAM_SOURCES if kernel == "k_ras_stream" else RAS_SOURCES)
+    traffic = ncu_traffic(key, sources)
+    limiter = (ncu_entry(key, sources) or {}).get("limiter")
     flops = FLOPS_PER_CELL_SWEEP * cells * sweeps_per_launch
     tflops = flops / avg_s / 1e12
     alu_peak = NOMINAL_FP32_TFLOPS if dt_name == "f32" else NOMINAL_FP64_TFLOPS
     hbm_min = min_bytes / avg_s / 1e9
     hbm_eff = eff_bytes / avg_s / 1e9
     peak_src = ("%s (MEASURED_PEAKS.json hbm_gbs)" % peak_kind) if peak_kind == "measured" else "fallback 6800 GB/s"
-    alu_bound = k > 1
+    alu_bound = k > 1 and kernel != "k_ras_stream"
     if alu_bound:
         roofline = {"bound": "alu", "achieved": tflops, "peak": alu_peak, "unit": "TFLOP/s", "frac": tflops / alu_peak,
                     "traffic": traffic,
@@ -453,7 +460,7 @@ def run_ours(args):
         roofline = {"bound": "hbm", "achieved": hbm_min, "peak": peak, "unit": "GB/s", "frac": hbm_min / peak,
                     "traffic": traffic, "peak_source": peak_src, "algorithmic_bytes_per_launch": min_bytes}
     roofline.update({
-        "kernel": tile_kernel_name(api, n, args.tile, o, dt_name), "kernel_avg_ms": avg_ms,
+        "kernel": kernel, "kernel_avg_ms": avg_ms,
         "kernel_share": ras_ms / ms_total, "sweeps_per_launch": sweeps_per_launch,
         "flops_per_cell_sweep": FLOPS_PER_CELL_SWEEP, "limiter": limiter,
         "traffic_note": "traffic = dram__bytes_read.sum + dram__bytes_write.sum per launch from the committed "

@@ -123,6 +123,14 @@ struct RasRun {
 template <typename T>
 cudaError_t launch_ras(const GridDesc<T> &g, const Coeffs<T> &c, T omega, const TileGrid &tg, int ksweeps,
                        int overlap, const T *vx, const T *vy, T *ox, T *oy, const RasRun &run, cudaStream_t s);
+// Row-streaming form of a RAS schedule that equals global Jacobi (FP32,
+// stream_kernels.cu): the number of passes that `sweeps` sweeps take (near
+// equal shares of them each), 0 where the tile kernels run it instead, and one
+// pass of `sweeps` sweeps from (vx, vy) to the unknowns of (ox, oy).
+int stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run);
+cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
+                              const float *vx, const float *vy, float *ox, float *oy, const RasRun &run,
+                              cudaStream_t s);
 // shared memory a RAS launch needs for this grid, tile and overlap
 size_t ras_smem_bytes(int nx, int ny, int ti, int tj, int overlap, size_t elem);
 // Whether a Jacobi-equivalent smoothing of an nx x ny level runs all its sweeps
@@ -242,7 +250,8 @@ template <typename T>
 int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx, T *sy, const SmoothSpec &p,
                    const RasRun &run, cudaStream_t s, LaunchHook &hook, bool *swapped = nullptr, T *tx = nullptr,
                    T *ty = nullptr);
-// ping-pong passes of one smoothing call (0 for RBGS, which works in place)
-int smooth_passes(const SmoothSpec &p);
+// ping-pong passes of one smoothing call
+template <typename T>
+int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run);
 
 } // namespace stokes

@@ -6,11 +6,27 @@
 
 namespace stokes {
 
+namespace {
+
+// passes of the row-streaming kernel for this smoothing, 0 if it does not take
+// it: a RAS schedule with overlap >= k - 1 is global Jacobi in any traversal
+template <typename T>
+int stream_passes_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
+{
+    if constexpr (sizeof(T) == 4)
+        return p.variant == STOKES_RAS && p.overlap >= p.k - 1 ? stream_passes(g, p.sweeps, run) : 0;
+    return 0;
+}
+
+} // namespace
+
 // number of ping-pong passes of a smoothing (one per sweep; one per outer
-// iteration of RAS)
-int smooth_passes(const SmoothSpec &p)
+// iteration of RAS, or per pass of the row-streaming kernel)
+template <typename T>
+int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
 {
     if (p.sweeps <= 0) return 0;
+    if (const int n = stream_passes_of(g, p, run)) return n;
     if (p.variant == STOKES_RAS) return (p.sweeps + p.k - 1) / p.k;
     return p.sweeps;
 }
@@ -33,7 +49,7 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     // and an odd number n >= 3 of passes, pass 1 goes from (vx, vy) to (sx, sy),
     // passes 2 .. n-1 alternate between the two scratch pairs and pass n
     // writes (vx, vy): the result lands in place without a copy back.
-    const int n_pass = smooth_passes(p);
+    const int n_pass = smooth_passes(g, p, run);
     const bool three = tx && ty && !swapped && n_pass >= 3 && (n_pass & 1);
     T *ax = vx, *ay = vy, *bx = sx, *by = sy;
     LAUNCH(STOKES_K_COPY, 1, launch_copy_walls<T>(g, vx, vy, sx, sy, s));
@@ -55,7 +71,23 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
         ax = nx_;
         ay = ny_;
     };
-    if (p.variant == STOKES_RAS) {
+    const int n_stream = stream_passes_of(g, p, run);
+    if (n_stream > 0) {
+        if constexpr (sizeof(T) == 4) {
+            const int n_outer = (p.sweeps + p.k - 1) / p.k;
+            if (p.shift_mode == STOKES_SHIFT_LIST) // the shifts change nothing, but bad ones stay refused
+                for (int t = 0; t < n_outer; ++t)
+                    if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 ||
+                        p.shifts[2 * t + 1] >= p.tj)
+                        return STOKES_ERR_ARG;
+            for (int t = 0; t < n_stream; ++t) {
+                const int ks = p.sweeps / n_stream + (t < p.sweeps % n_stream ? 1 : 0);
+                LAUNCH(STOKES_K_RAS, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, run, s));
+                ++passes;
+                advance();
+            }
+        }
+    } else if (p.variant == STOKES_RAS) {
         const int n_outer = (p.sweeps + p.k - 1) / p.k;
         for (int t = 0; t < n_outer; ++t) {
             const int ks = (t == n_outer - 1) ? p.sweeps - (n_outer - 1) * p.k : p.k;
@@ -98,6 +130,8 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     return STOKES_OK;
 }
 
+template int smooth_passes<float>(const GridDesc<float> &, const SmoothSpec &, const RasRun &);
+template int smooth_passes<double>(const GridDesc<double> &, const SmoothSpec &, const RasRun &);
 template int smooth_buffers<float>(const GridDesc<float> &, const Coeffs<float> &, float *, float *, float *,
                                    float *, const SmoothSpec &, const RasRun &, cudaStream_t, LaunchHook &, bool *,
                                    float *, float *);

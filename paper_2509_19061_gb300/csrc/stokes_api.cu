@@ -267,11 +267,26 @@ int smooth_impl(stokes_ctx *c, T *vx, T *vy, const stokes_smooth_params *p, int 
         k.by = (const T *)c->fy;
     }
     const SmoothSpec spec = spec_of(p, ti, tj);
-    const int n_pass = smooth_passes(spec);
+    const int n_pass = smooth_passes(grid_of<T>(c), spec, run_opts(c));
     if (n_pass >= 3 && (n_pass & 1) && !c->sx2) { // second scratch pair: odd pass counts end in place
-        int st = alloc_field(c, &c->sx2);
-        if (st == STOKES_OK) st = alloc_field(c, &c->sy2);
-        if (st != STOKES_OK) return st;
+        // A schedule whose own outer iterations would not need the pair (the
+        // row-streaming kernel's passes do) ends with a copy instead where it
+        // cannot be had: under stream capture, or out of memory.
+        const int own = spec.variant == STOKES_RAS ? (spec.sweeps + spec.k - 1) / spec.k : n_pass;
+        const bool optional = own < 3 || !(own & 1);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (optional && cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+        if (!optional || cap == cudaStreamCaptureStatusNone) {
+            int st = alloc_field(c, &c->sx2);
+            if (st == STOKES_OK) st = alloc_field(c, &c->sy2);
+            if (st != STOKES_OK) {
+                cudaFree(c->sx2);
+                cudaFree(c->sy2);
+                c->sx2 = c->sy2 = nullptr;
+                if (!optional || st != STOKES_ERR_OOM) return st;
+                cudaGetLastError();
+            }
+        }
     }
     return smooth_buffers<T>(grid_of<T>(c), k, vx, vy, (T *)c->sx, (T *)c->sy, spec, run_opts(c), c->stream, hook,
                              nullptr, (T *)c->sx2, (T *)c->sy2);
