@@ -990,7 +990,8 @@ def variant_table(args, api, prob):
         out[label] = {"gcell_updates_per_s": cu / 1e9, "effective_gbs": gbs, "frac": gbs / peak,
                       "sweeps": kw["sweeps"], "ms_per_call": ms}
         if kw["variant"] in ("ras", "blocked"):
-            out[label]["kernel"] = tile_kernel_name(api, n, kw["tile"], kw.get("overlap", 0), dt_name)
+            # (blocked Jacobi always runs the tile kernel)
+            out[label]["kernel"] = tile_kernel_name(api, n, kw["tile"], kw.get("k", 2), kw.get("overlap", 0), dt_name)
     for c, _, _ in ctxs.values():
         c.close()
     return out

@@ -199,9 +199,9 @@ int stokes_apply_operator(stokes_ctx *ctx, const void *vx, const void *vy, const
  * (Sec. 5).  p may be NULL (p = 0).  Requires stokes_set_viscosity and
  * stokes_set_rhs.  Asynchronous.  The passes ping-pong between (vx, vy) and
  * context-owned scratch fields; the first call whose pass count is odd and at
- * least 3 (RAS: ceil(sweeps / k) outer iterations, or the passes of up to
- * eight sweeps that a large FP32 schedule with o >= k - 1 runs instead;
- * Jacobi variants: one pass per sweep) allocates a second scratch pair (two fields) so that the result
+ * least 3 (RAS: ceil(sweeps / k) outer iterations, Jacobi variants:
+ * one pass per sweep; large FP32 schedules with o >= k - 1, and fused Jacobi,
+ * run passes of up to eight sweeps instead) allocates a second scratch pair (two fields) so that the result
  * ends in (vx, vy) without a copy: make that call once before capturing
  * stokes_smooth into a CUDA graph.  Returns STOKES_ERR_OOM if that allocation
  * fails. */

@@ -9,12 +9,16 @@ namespace stokes {
 namespace {
 
 // passes of the row-streaming kernel for this smoothing, 0 if it does not take
-// it: a RAS schedule with overlap >= k - 1 is global Jacobi in any traversal
+// it: a RAS schedule with overlap >= k - 1 is global Jacobi in any traversal,
+// and fused Jacobi's sweeps need not each cross the grid before the next
+// begins (20 sweeps of 4001 x 2999: 408 us, 1822 us as 20 passes of
+// k_jacobi_rows).  Separate-pass and blocked Jacobi keep their own passes.
 template <typename T>
 int stream_passes_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
 {
     if constexpr (sizeof(T) == 4)
-        return p.variant == STOKES_RAS && p.overlap >= p.k - 1 ? stream_passes(g, p.sweeps, run) : 0;
+        if ((p.variant == STOKES_RAS && p.overlap >= p.k - 1) || p.variant == STOKES_JACOBI_FUSED)
+            return stream_passes(g, p.sweeps, run);
     return 0;
 }
 
@@ -74,15 +78,16 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     const int n_stream = stream_passes_of(g, p, run);
     if (n_stream > 0) {
         if constexpr (sizeof(T) == 4) {
-            const int n_outer = (p.sweeps + p.k - 1) / p.k;
-            if (p.shift_mode == STOKES_SHIFT_LIST) // the shifts change nothing, but bad ones stay refused
+            const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + p.k - 1) / p.k : 0;
+            const int kind = p.variant == STOKES_RAS ? STOKES_K_RAS : STOKES_K_JACOBI;
+            if (p.variant == STOKES_RAS && p.shift_mode == STOKES_SHIFT_LIST) // the shifts change nothing, but bad ones stay refused
                 for (int t = 0; t < n_outer; ++t)
                     if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 ||
                         p.shifts[2 * t + 1] >= p.tj)
                         return STOKES_ERR_ARG;
             for (int t = 0; t < n_stream; ++t) {
                 const int ks = p.sweeps / n_stream + (t < p.sweeps % n_stream ? 1 : 0);
-                LAUNCH(STOKES_K_RAS, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, run, s));
+                LAUNCH(kind, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, run, s));
                 ++passes;
                 advance();
             }

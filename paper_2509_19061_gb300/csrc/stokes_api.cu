@@ -272,7 +272,7 @@ int smooth_impl(stokes_ctx *c, T *vx, T *vy, const stokes_smooth_params *p, int 
         // A schedule whose own outer iterations would not need the pair (the
         // row-streaming kernel's passes do) ends with a copy instead where it
         // cannot be had: under stream capture, or out of memory.
-        const int own = spec.variant == STOKES_RAS ? (spec.sweeps + spec.k - 1) / spec.k : n_pass;
+        const int own = spec.variant == STOKES_RAS ? (spec.sweeps + spec.k - 1) / spec.k : spec.sweeps;
         const bool optional = own < 3 || !(own & 1);
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (optional && cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();

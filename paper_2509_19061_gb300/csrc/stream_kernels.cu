@@ -1,6 +1,6 @@
 // stream_kernels.cu -- temporally blocked Jacobi by row streaming, the FP32
-// path of RAS schedules that equal global Jacobi (overlap >= k - 1, Sec. 4.3)
-// on grids large enough to fill the GPU.
+// path of fused Jacobi and of RAS schedules that equal global Jacobi
+// (overlap >= k - 1, Sec. 4.3) on grids large enough to fill the GPU.
 //
 // Such a schedule's result does not depend on its tiles, so any traversal that
 // performs the same sweeps gives the same values.  The tile kernels sweep the
