@@ -104,6 +104,17 @@ template <typename T>
 cudaError_t launch_energy_raw(const GridDesc<T> &g, const T *eta_c, const T *eta_n, const T *fx, const T *fy,
                               const T *p, const T *vx, const T *vy, double *partials, double *out, cudaStream_t s);
 
+// ---- FP64 operator by row-marching warps (op_rows.cu) ---------------------
+// Whether a grid is large enough for it; every buffer it gets starts on a
+// 16-byte boundary.
+bool op_rows_takes(int nx, int ny);
+// M v + G p at the unknowns, zero elsewhere (p may be NULL)
+cudaError_t op_rows_apply(const GridDesc<double> &g, const double *ec, const double *en, const double *vx,
+                          const double *vy, const double *p, double *ox, double *oy, cudaStream_t s);
+// r = b - M v at the unknowns, zero on the walls
+cudaError_t op_rows_residual(const GridDesc<double> &g, const double *ec, const double *en, const double *bx,
+                             const double *by, const double *vx, const double *vy, double *rx, double *ry,
+                             cudaStream_t s);
 // ---- tiled / RAS kernel (ras_kernels.cu) ---------------------------------
 struct TileGrid {
     int ti, tj;   // tile size (cells)

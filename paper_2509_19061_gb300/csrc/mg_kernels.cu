@@ -410,6 +410,10 @@ template <typename T>
 cudaError_t mg_residual(const MgLevel &l, cudaStream_t s)
 {
     const GridDesc<T> g = make_grid<T>(l.nx, l.ny, l.pitch, l.hx, l.hy);
+    if constexpr (sizeof(T) == 8)
+        if (op_rows_takes(l.nx, l.ny))
+            return op_rows_residual(g, (const T *)l.ec, (const T *)l.en, (const T *)l.bx, (const T *)l.by,
+                                    (const T *)l.vx, (const T *)l.vy, (T *)l.rx, (T *)l.ry, s);
     k_residual<T><<<grid2d(l.nx + 1, l.ny + 1), dim3(BX, BY), 0, s>>>(g, (const T *)l.ec, (const T *)l.en,
                                                                        (const T *)l.bx, (const T *)l.by,
                                                                        (const T *)l.vx, (const T *)l.vy, (T *)l.rx,

@@ -500,6 +500,12 @@ template <typename T>
 cudaError_t launch_apply(const GridDesc<T> &g, const T *eta_c, const T *eta_n, const T *vx, const T *vy, const T *p,
                          T *ox, T *oy, cudaStream_t s)
 {
+    if constexpr (sizeof(T) == 8) {
+        // (the caller's buffers need not be aligned for the row kernel's 16-byte loads)
+        const uintptr_t all = (uintptr_t)vx | (uintptr_t)vy | (uintptr_t)p | (uintptr_t)ox | (uintptr_t)oy;
+        if (op_rows_takes(g.nx, g.ny) && (all & 15u) == 0)
+            return op_rows_apply(g, eta_c, eta_n, vx, vy, p, ox, oy, s);
+    }
     k_apply<T><<<grid2d(g.pitch, g.ny + 1), dim3(BX, BY), 0, s>>>(g, eta_c, eta_n, vx, vy, p, ox, oy);
     return cudaGetLastError();
 }

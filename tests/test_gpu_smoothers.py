@@ -178,6 +178,32 @@ def test_entry_points_reject_buffers_off_16_byte_boundaries(api, dtype):
     assert rp == 0.0 and ff > 0.0
 
 
+@pytest.mark.parametrize("nx,ny,square", [(359, 301, True), (360, 299, False), (418, 251, True), (1201, 90, False),
+                                          (5, 25000, True), (25000, 5, False)])
+@pytest.mark.parametrize("with_p", [False, True])
+def test_operator_f64_by_rows(api, nx, ny, square, with_p):
+    """M v + G p on grids the FP64 row kernel takes: strips of 60 columns that
+    end before, on and after the grid's edge, bands of many and of few rows;
+    buffers off 16-byte boundaries take the general kernel and agree."""
+    import torch
+    prob = rand_problem(nx, ny, 61, lx=1.0, ly=ny / nx if square else 0.8)
+    vx, vy = inputs.random_velocity(nx, ny, 62)
+    p = inputs.random_pressure(nx, ny, 63) if with_p else None
+    r = Run(api, prob, "f64", (vx, vy), p)
+    ox, oy = r.ctx.apply(r.vx, r.vy, r.p)
+    g = ogrid(prob)
+    want = ora.apply_M(g, vx, vy)
+    if with_p:
+        want = tuple(a + b for a, b in zip(want, ora.apply_G(g, p)))
+    assert rel((r.ctx.unpack(ox, "vx"), r.ctx.unpack(oy, "vy")), want) <= F64_TOL
+    assert float(ox[ny].abs().sum()) == 0.0 and float(oy[:, nx:].abs().sum()) == 0.0
+    off = lambda t: torch.cat([t.new_zeros(1), t.reshape(-1)])[1:].view(t.shape)  # noqa: E731
+    o2 = (off(torch.full_like(ox, 7.0)), off(torch.full_like(oy, 7.0)))
+    api.stokes_apply_operator(r.ctx.ctx, off(r.vx), off(r.vy), r.p, *o2)
+    for a, b in zip((ox, oy), o2):
+        assert float((a - b).abs().max()) <= 1e-15 * float(a.abs().max())
+
+
 def test_energy_norm_is_one_at_zero_state(api):
     prob = inputs.sinker_problem(64)
     r = Run(api, prob, "f64")
