@@ -142,6 +142,10 @@ int stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run);
 cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
                               const float *vx, const float *vy, float *ox, float *oy, const RasRun &run,
                               cudaStream_t s);
+// the same in FP64 (stream64_kernels.cu)
+int stream64_passes(const GridDesc<double> &g, int sweeps, const RasRun &run);
+cudaError_t launch_ras_stream64(const GridDesc<double> &g, const Coeffs<double> &c, double omega, int sweeps,
+                                const double *vx, const double *vy, double *ox, double *oy, cudaStream_t s);
 // shared memory a RAS launch needs for this grid, tile and overlap
 size_t ras_smem_bytes(int nx, int ny, int ti, int tj, int overlap, size_t elem);
 // Whether a Jacobi-equivalent smoothing of an nx x ny level runs all its sweeps

@@ -8,6 +8,12 @@ namespace stokes {
 
 namespace {
 
+// global Jacobi in any traversal: fused Jacobi, and RAS with overlap >= k - 1
+bool any_traversal(const SmoothSpec &p)
+{
+    return (p.variant == STOKES_RAS && p.overlap >= p.k - 1) || p.variant == STOKES_JACOBI_FUSED;
+}
+
 // passes of the row-streaming kernel for this smoothing, 0 if it does not take
 // it: a RAS schedule with overlap >= k - 1 is global Jacobi in any traversal,
 // and fused Jacobi's sweeps need not each cross the grid before the next
@@ -16,10 +22,9 @@ namespace {
 template <typename T>
 int stream_passes_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
 {
-    if constexpr (sizeof(T) == 4)
-        if ((p.variant == STOKES_RAS && p.overlap >= p.k - 1) || p.variant == STOKES_JACOBI_FUSED)
-            return stream_passes(g, p.sweeps, run);
-    return 0;
+    if (!any_traversal(p)) return 0;
+    if constexpr (sizeof(T) == 4) return stream_passes(g, p.sweeps, run);
+    else return stream64_passes(g, p.sweeps, run);
 }
 
 } // namespace
@@ -48,6 +53,13 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
         if (st != STOKES_OK) return st;                                                                            \
     } while (0)
     if (p.sweeps == 0) return STOKES_OK;
+    const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + p.k - 1) / p.k : 0;
+    const int n_stream = stream_passes_of(g, p, run);
+    const int kind = p.variant == STOKES_RAS ? STOKES_K_RAS : STOKES_K_JACOBI;
+    if (n_stream > 0 && p.variant == STOKES_RAS && p.shift_mode == STOKES_SHIFT_LIST)
+        for (int t = 0; t < n_outer; ++t) // the shifts change nothing, but bad ones stay refused
+            if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 || p.shifts[2 * t + 1] >= p.tj)
+                return STOKES_ERR_ARG;
     // ping-pong between (vx, vy) and the scratch pair; the scratch walls take
     // the Dirichlet values of (vx, vy).  With a second scratch pair (tx, ty)
     // and an odd number n >= 3 of passes, pass 1 goes from (vx, vy) to (sx, sy),
@@ -75,25 +87,17 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
         ax = nx_;
         ay = ny_;
     };
-    const int n_stream = stream_passes_of(g, p, run);
     if (n_stream > 0) {
-        if constexpr (sizeof(T) == 4) {
-            const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + p.k - 1) / p.k : 0;
-            const int kind = p.variant == STOKES_RAS ? STOKES_K_RAS : STOKES_K_JACOBI;
-            if (p.variant == STOKES_RAS && p.shift_mode == STOKES_SHIFT_LIST) // the shifts change nothing, but bad ones stay refused
-                for (int t = 0; t < n_outer; ++t)
-                    if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 ||
-                        p.shifts[2 * t + 1] >= p.tj)
-                        return STOKES_ERR_ARG;
-            for (int t = 0; t < n_stream; ++t) {
-                const int ks = p.sweeps / n_stream + (t < p.sweeps % n_stream ? 1 : 0);
+        for (int t = 0; t < n_stream; ++t) {
+            const int ks = p.sweeps / n_stream + (t < p.sweeps % n_stream ? 1 : 0);
+            if constexpr (sizeof(T) == 4)
                 LAUNCH(kind, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, run, s));
-                ++passes;
-                advance();
-            }
+            else
+                LAUNCH(kind, 1, launch_ras_stream64(g, k, omega, ks, ax, ay, bx, by, s));
+            ++passes;
+            advance();
         }
     } else if (p.variant == STOKES_RAS) {
-        const int n_outer = (p.sweeps + p.k - 1) / p.k;
         for (int t = 0; t < n_outer; ++t) {
             const int ks = (t == n_outer - 1) ? p.sweeps - (n_outer - 1) * p.k : p.k;
             int si = 0, sj = 0;

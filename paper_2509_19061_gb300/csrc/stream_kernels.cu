@@ -303,7 +303,7 @@ void (*pick_stream(bool odd, bool square))(StreamArgs)
 
 int stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run)
 {
-    if (!run.allow_tma || run.pair_mode < 1 || sweeps < ST_MIN_SWEEPS) return 0;
+    if (!run.allow_tma || run.pair_mode != 1 || sweeps < ST_MIN_SWEEPS) return 0;
     // Below this a segment's 2 n extra rows outweigh the tiles' halo: 40 sweeps
     // take 101 us either way at 768^2, 80 (48 x 64 tiles: 70) at 512^2 and 111
     // (132) at 1024^2.

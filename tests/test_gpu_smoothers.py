@@ -708,6 +708,30 @@ def test_row_streaming_equals_global_jacobi(api, nx, ny, sweeps, square):
         assert np.array_equal(outs[0][0], outs[-1][0]) and np.array_equal(outs[0][1], outs[-1][1])
 
 
+@pytest.mark.parametrize("nx,ny,sweeps,square", [
+    (500, 300, 2, True), (559, 301, 3, False), (560, 299, 4, True), (561, 200, 5, False), (600, 180, 9, True),
+    (3, 40000, 4, False), (40000, 3, 7, True),
+])
+def test_row_streaming_f64_equals_global_jacobi(api, nx, ny, sweeps, square):
+    """The FP64 form: strips of 56 or 60 columns that end on, before and after
+    the grid's edge, chains of two to four warps, short segments, with a
+    pressure, moving walls and NaN in the padding."""
+    prob = rand_problem(nx, ny, 55, lx=1.0, ly=ny / nx if square else 0.7)
+    vx, vy = inputs.random_velocity(nx, ny, 56, 0.1)
+    vx[:, 0], vx[:, nx], vy[0], vy[ny] = 0.3, -0.2, 0.1, 0.4
+    p = inputs.random_pressure(nx, ny, 57)
+    outs = []
+    for kw in (dict(variant="jacobi"), dict(variant="ras", tile=(16, 16), k=2, overlap=1, seed=82),
+               dict(variant="fused")):
+        r = Run(api, prob, "f64", (vx, vy), p)
+        r.vx, r.vy = _with_canaries(api, r.ctx, r.vx, "vx"), _with_canaries(api, r.ctx, r.vy, "vy")
+        r.smooth(sweeps=sweeps, **kw)
+        outs.append(r.v())
+        assert np.isnan(r.vx.cpu().numpy()[ny:]).all()
+        r.ctx.close()
+        assert np.array_equal(outs[0][0], outs[-1][0]) and np.array_equal(outs[0][1], outs[-1][1])
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("kw", [
     dict(variant="jacobi", sweeps=3), dict(variant="fused", sweeps=3), dict(variant="rbgs", sweeps=2),
