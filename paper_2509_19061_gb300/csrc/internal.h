@@ -146,6 +146,14 @@ cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, 
 int stream64_passes(const GridDesc<double> &g, int sweeps, const RasRun &run);
 cudaError_t launch_ras_stream64(const GridDesc<double> &g, const Coeffs<double> &c, double omega, int sweeps,
                                 const double *vx, const double *vy, double *ox, double *oy, cudaStream_t s);
+// All sweeps of a small grid's damped Jacobi in one launch, in place
+// (cluster_kernels.cu): whether a smoothing of `sweeps` sweeps takes it, and
+// the launch.
+template <typename T>
+bool cluster_takes(int nx, int ny, int sweeps, const RasRun &run);
+template <typename T>
+cudaError_t launch_jacobi_cluster(const GridDesc<T> &g, const Coeffs<T> &c, T omega, int sweeps, T *vx, T *vy,
+                                  cudaStream_t s);
 // shared memory a RAS launch needs for this grid, tile and overlap
 size_t ras_smem_bytes(int nx, int ny, int ti, int tj, int overlap, size_t elem);
 // Whether a Jacobi-equivalent smoothing of an nx x ny level runs all its sweeps

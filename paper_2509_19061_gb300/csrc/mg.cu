@@ -158,7 +158,7 @@ int build(MgHierarchy *h, const MgOuter &o, int levels, int coarsest, cudaStream
 }
 
 // smoothing spec of level l and phase ph
-SmoothSpec level_spec(const stokes_mg_params *p, const MgLevel &l, int lvl, int ph, size_t es)
+SmoothSpec level_spec(const stokes_mg_params *p, const MgLevel &l, int lvl, int ph, size_t es, const RasRun &run)
 {
     const stokes_smooth_params sm = level_smoother(p->smoother, lvl);
     SmoothSpec s;
@@ -173,12 +173,19 @@ SmoothSpec level_spec(const stokes_mg_params *p, const MgLevel &l, int lvl, int 
     s.shift_mode = STOKES_SHIFT_SPLITMIX;
     s.shifts = nullptr;
     // Jacobi in any schedule (and RAS with overlap >= k-1, which is Jacobi)
-    // on a level whose whole-level window fits a register tile kernel: all
-    // sweeps in one launch (the same map, so the same values)
+    // on a level that a cluster of CTAs holds, or whose whole-level window fits
+    // a register tile kernel: all sweeps in one launch (the same map, so the
+    // same values).  FP32 prefers the tile (40 sweeps of 32^2: 15.6 us, 26 by a
+    // cluster), FP64 the cluster's many FP64 pipes (52 us, 190 on one SM).
     const bool jacobi = sm.variant == STOKES_JACOBI || sm.variant == STOKES_JACOBI_FUSED ||
                         sm.variant == STOKES_JACOBI_BLOCKED ||
                         (sm.variant == STOKES_RAS && sm.overlap >= sm.k - 1);
-    if (jacobi && s.sweeps > 0 && ras_whole_level_tile(l.nx, l.ny, es)) {
+    const bool tile = ras_whole_level_tile(l.nx, l.ny, es);
+    const bool cluster = es == 8 ? cluster_takes<double>(l.nx, l.ny, s.sweeps, run)
+                                 : !tile && cluster_takes<float>(l.nx, l.ny, s.sweeps, run);
+    if (jacobi && cluster) {
+        s.variant = STOKES_JACOBI_FUSED; // all sweeps by a cluster of CTAs
+    } else if (jacobi && s.sweeps > 0 && tile) {
         s.variant = STOKES_RAS;
         s.ti = l.nx;
         s.tj = l.ny;
@@ -230,7 +237,8 @@ int enqueue_precond(MgHierarchy *h, const Tc *rx, const Tc *ry, Tc *zx, Tc *zy, 
     auto smooth_level = [&](MgLevel &f, int l, int phase) -> int {
         bool swapped = false;
         const int r = smooth_buffers<Ti>(level_grid<Ti>(f), level_coeffs<Ti>(f), (Ti *)f.vx, (Ti *)f.vy, (Ti *)f.sx,
-                                         (Ti *)f.sy, level_spec(p, f, l, phase, sizeof(Ti)), run, s, hook, &swapped);
+                                         (Ti *)f.sy, level_spec(p, f, l, phase, sizeof(Ti), run), run, s, hook,
+                                         &swapped);
         if (swapped) {
             std::swap(f.vx, f.sx);
             std::swap(f.vy, f.sy);

@@ -14,6 +14,12 @@ bool any_traversal(const SmoothSpec &p)
     return (p.variant == STOKES_RAS && p.overlap >= p.k - 1) || p.variant == STOKES_JACOBI_FUSED;
 }
 
+template <typename T>
+bool takes_cluster(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
+{
+    return any_traversal(p) && cluster_takes<T>(g.nx, g.ny, p.sweeps, run);
+}
+
 // passes of the row-streaming kernel for this smoothing, 0 if it does not take
 // it: a RAS schedule with overlap >= k - 1 is global Jacobi in any traversal,
 // and fused Jacobi's sweeps need not each cross the grid before the next
@@ -35,6 +41,7 @@ template <typename T>
 int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
 {
     if (p.sweeps <= 0) return 0;
+    if (takes_cluster(g, p, run)) return 1;
     if (const int n = stream_passes_of(g, p, run)) return n;
     if (p.variant == STOKES_RAS) return (p.sweeps + p.k - 1) / p.k;
     return p.sweeps;
@@ -54,12 +61,17 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     } while (0)
     if (p.sweeps == 0) return STOKES_OK;
     const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + p.k - 1) / p.k : 0;
+    const bool cluster = takes_cluster(g, p, run);
     const int n_stream = stream_passes_of(g, p, run);
     const int kind = p.variant == STOKES_RAS ? STOKES_K_RAS : STOKES_K_JACOBI;
-    if (n_stream > 0 && p.variant == STOKES_RAS && p.shift_mode == STOKES_SHIFT_LIST)
+    if ((cluster || n_stream > 0) && p.variant == STOKES_RAS && p.shift_mode == STOKES_SHIFT_LIST)
         for (int t = 0; t < n_outer; ++t) // the shifts change nothing, but bad ones stay refused
             if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 || p.shifts[2 * t + 1] >= p.tj)
                 return STOKES_ERR_ARG;
+    if (cluster) {
+        LAUNCH(kind, 1, launch_jacobi_cluster<T>(g, k, omega, p.sweeps, vx, vy, s));
+        return STOKES_OK;
+    }
     // ping-pong between (vx, vy) and the scratch pair; the scratch walls take
     // the Dirichlet values of (vx, vy).  With a second scratch pair (tx, ty)
     // and an odd number n >= 3 of passes, pass 1 goes from (vx, vy) to (sx, sy),

@@ -708,6 +708,33 @@ def test_row_streaming_equals_global_jacobi(api, nx, ny, sweeps, square):
         assert np.array_equal(outs[0][0], outs[-1][0]) and np.array_equal(outs[0][1], outs[-1][1])
 
 
+@pytest.mark.parametrize("dtype,nx,ny", [
+    ("f32", 2, 2), ("f32", 33, 31), ("f32", 64, 64), ("f32", 128, 128), ("f32", 256, 9), ("f32", 9, 256), ("f32", 31, 500),
+    ("f64", 2, 2), ("f64", 5, 3), ("f64", 32, 32), ("f64", 33, 47), ("f64", 72, 64), ("f64", 250, 18), ("f64", 18, 250),
+])
+@pytest.mark.parametrize("square", [True, False])
+def test_cluster_equals_global_jacobi(api, dtype, nx, ny, square):
+    """Small grids run all sweeps of a schedule with o >= k - 1, and of fused
+    Jacobi, in one cluster of CTAs: bands of one to many rows, partly filled
+    and empty bands, one to eight rows per thread; with moving walls, value
+    for value the separate-pass Jacobi, walls and padding untouched."""
+    prob = rand_problem(nx, ny, 71, lx=1.0, ly=ny / nx if square else 0.7)
+    vx, vy = inputs.random_velocity(nx, ny, 72, 0.1)
+    vx[:, 0], vx[:, nx], vy[0], vy[ny] = 0.3, -0.2, 0.1, 0.4
+    p = inputs.random_pressure(nx, ny, 73)
+    for sweeps in (2, 7):
+        outs = []
+        for kw in (dict(variant="jacobi"), dict(variant="ras", tile=(16, 16), k=2, overlap=1, seed=81),
+                   dict(variant="fused")):
+            r = Run(api, prob, dtype, (vx, vy), p)
+            r.vx, r.vy = _with_canaries(api, r.ctx, r.vx, "vx"), _with_canaries(api, r.ctx, r.vy, "vy")
+            r.smooth(sweeps=sweeps, **kw)
+            outs.append(r.v())
+            assert np.isnan(r.vx.cpu().numpy()[ny:]).all()
+            r.ctx.close()
+            assert np.array_equal(outs[0][0], outs[-1][0]) and np.array_equal(outs[0][1], outs[-1][1])
+
+
 @pytest.mark.parametrize("nx,ny,sweeps,square", [
     (500, 300, 2, True), (559, 301, 3, False), (560, 299, 4, True), (561, 200, 5, False), (600, 180, 9, True),
     (3, 40000, 4, False), (40000, 3, 7, True),
