@@ -143,6 +143,14 @@ struct TileLaunch {
     bool square;      // every instance has square cells
 };
 
+// one pass of the row-streaming kernel over a group's square or other grids
+struct StreamLaunch {
+    const StreamEntry *tab;
+    const StreamTask *tasks;
+    int ntasks, sweeps;
+    bool square;
+};
+
 // one instance of a group: level grid and coefficients, velocity and scratch
 template <typename T>
 struct GInst {
@@ -156,6 +164,7 @@ struct GInst {
 template <typename T>
 struct Group {
     std::vector<TileLaunch<T>> launches;
+    std::vector<StreamLaunch> streams; // instead of `launches` (FP32, overlap >= k - 1)
     const BLevel<T> *lev = nullptr; // vx, vy, sx, sy per instance (copies)
     Sub sub;                        // the instances over (nx+1) x (ny+1), a tall map
     bool walls = false, back = false;
@@ -182,6 +191,16 @@ int plan_group(Owned &o, const std::vector<GInst<T>> &gi, const RasForm &f, bool
         ay[q] = gi[q].vy;
         bx[q] = gi[q].sx;
         by[q] = gi[q].sy;
+    }
+    // a schedule that equals global Jacobi runs by row streaming, as in smooth_buffers
+    int n_stream = 0;
+    if (sizeof(T) == 4 && !single && f.overlap >= f.k - 1) {
+        long long cells = 0;
+        for (const GInst<T> &x : gi) cells += (long long)x.g.nx * x.g.ny;
+        RasRun r{};
+        r.allow_tma = tma;
+        r.pair_mode = pair_mode;
+        n_stream = stream_batch_passes(cells, f.sweeps, r);
     }
     const int n_outer = (f.sweeps + f.k - 1) / f.k;
     for (int t = 0; t < n_outer; ++t) {
@@ -219,6 +238,7 @@ int plan_group(Owned &o, const std::vector<GInst<T>> &gi, const RasForm &f, bool
         // a TMA-staged shape (one-column or pair layout) fits by construction
         const bool staged = tma && ras_batched_tma(shi, shj, ov, sizeof(T), pair_mode);
         if (!staged && ras_batched_smem_bytes(shi, shj, ov, sizeof(T)) > (size_t)ras_max_smem()) return STOKES_ERR_ARG;
+        if (n_stream > 0) continue; // (refused as the tile launches would be)
         TileLaunch<T> L;
         ST(upload(o, tab, &L.tab, s));
         {
@@ -246,7 +266,43 @@ int plan_group(Owned &o, const std::vector<GInst<T>> &gi, const RasForm &f, bool
         L.overlap = ov;
         out->launches.push_back(L);
     }
-    out->back = (n_outer & 1) != 0;
+    out->back = ((n_stream > 0 ? n_stream : n_outer) & 1) != 0;
+    if constexpr (sizeof(T) == 4) {
+        for (size_t q = 0; q < n && n_stream > 0; ++q) { // from the start (the loop above swapped the buffers)
+            ax[q] = gi[q].vx;
+            ay[q] = gi[q].vy;
+            bx[q] = gi[q].sx;
+            by[q] = gi[q].sy;
+        }
+        for (int t = 0; t < n_stream; ++t) {
+            const int ks = f.sweeps / n_stream + (t < f.sweeps % n_stream ? 1 : 0);
+            std::vector<StreamEntry> es[2]; // square cells and others
+            for (size_t q = 0; q < n; ++q) {
+                StreamEntry e = stream_entry(gi[q].g, gi[q].c, out->omega, ks, ax[q], ay[q], bx[q], by[q]);
+                e.inst = gi[q].inst;
+                es[gi[q].g.square ? 0 : 1].push_back(e);
+                std::swap(ax[q], bx[q]);
+                std::swap(ay[q], by[q]);
+            }
+            for (int w = 0; w < 2; ++w) {
+                if (es[w].empty()) continue;
+                StreamLaunch L;
+                L.ntasks = stream_split(es[w].data(), (int)es[w].size());
+                L.sweeps = ks;
+                L.square = w == 0;
+                std::vector<StreamTask> tasks;
+                for (int q = 0; q < (int)es[w].size(); ++q)
+                    for (int u = 0; u < es[w][q].strips * es[w][q].segs; ++u) tasks.push_back({q, u});
+                // the longest first: the last CTAs to start are then the short ones
+                std::stable_sort(tasks.begin(), tasks.end(), [&](const StreamTask &x, const StreamTask &y) {
+                    return es[w][x.entry].rows > es[w][y.entry].rows;
+                });
+                ST(upload(o, es[w], &L.tab, s));
+                ST(upload(o, tasks, &L.tasks, s));
+                out->streams.push_back(L);
+            }
+        }
+    }
     return STOKES_OK;
 }
 
@@ -254,7 +310,7 @@ int plan_group(Owned &o, const std::vector<GInst<T>> &gi, const RasForm &f, bool
 template <typename T>
 int run_group(const Group<T> &G, const int *live, const RasRun &run, cudaStream_t s, long long *nk)
 {
-    if (G.launches.empty()) return STOKES_OK;
+    if (G.launches.empty() && G.streams.empty()) return STOKES_OK;
     if (G.walls) {
         CK(batch_copy_walls<T>(G.lev, G.sub.map, G.sub.nseg, live, s));
         ++*nk;
@@ -262,6 +318,10 @@ int run_group(const Group<T> &G, const int *live, const RasRun &run, cudaStream_
     for (const TileLaunch<T> &L : G.launches) {
         CK(launch_ras_batched<T>(L.tab, L.tmap, L.maps, L.count, L.total, L.ti, L.tj, L.ks, L.overlap, G.omega, live,
                                  run, L.square, s));
+        ++*nk;
+    }
+    for (const StreamLaunch &L : G.streams) {
+        CK(launch_ras_stream_batch(L.tab, L.tasks, L.ntasks, L.sweeps, L.square, live, s));
         ++*nk;
     }
     if (G.back) {

@@ -140,12 +140,41 @@ cudaError_t launch_ras(const GridDesc<T> &g, const Coeffs<T> &c, T omega, const 
 // pass of `sweeps` sweeps from (vx, vy) to the unknowns of (ox, oy).
 int stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run);
 cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
-                              const float *vx, const float *vy, float *ox, float *oy, const RasRun &run,
-                              cudaStream_t s);
+                              const float *vx, const float *vy, float *ox, float *oy, cudaStream_t s);
+
 // the same in FP64 (stream64_kernels.cu)
 int stream64_passes(const GridDesc<double> &g, int sweeps, const RasRun &run);
 cudaError_t launch_ras_stream64(const GridDesc<double> &g, const Coeffs<double> &c, double omega, int sweeps,
                                 const double *vx, const double *vy, double *ox, double *oy, cudaStream_t s);
+
+constexpr int ST_FIELDS = 8; // vx, vy, eta_c, eta_n, bx, by, 1/dx, 1/dy
+// one grid's share of a streaming pass
+struct StreamEntry {
+    GridDesc<float> g;
+    const float *f[ST_FIELDS];
+    float omega;
+    float *ox, *oy;
+    int sweeps;       // of the pass
+    int strips, segs; // column strips and row segments: one pair of warps each
+    int rows;         // cell rows per segment
+    int hl, own;      // columns left of the owned ones, and owned columns, of a strip
+    int inst;         // index into a batch's `live` flags
+};
+// entry and segment number (segment * strips + strip) of one pair of warps
+struct StreamTask {
+    int entry, part;
+};
+StreamEntry stream_entry(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps, const float *vx,
+                         const float *vy, float *ox, float *oy);
+// Splits the rows of `n` entries into segments for one launch; returns the
+// number of tasks (the sum of strips x segs).
+int stream_split(StreamEntry *e, int n);
+// Passes of a batch over `cells` cells altogether, as stream_passes.
+int stream_batch_passes(long long cells, int sweeps, const RasRun &run);
+// One pass over the tasks of a batch (device tables), all of `sweeps` sweeps
+// and square or not; entries whose live[inst] is 0 are skipped.
+cudaError_t launch_ras_stream_batch(const StreamEntry *tab, const StreamTask *tasks, int ntasks, int sweeps,
+                                    bool square, const int *live, cudaStream_t s);
 // All sweeps of a small grid's damped Jacobi in one launch, in place
 // (cluster_kernels.cu): whether a smoothing of `sweeps` sweeps takes it, and
 // the launch.

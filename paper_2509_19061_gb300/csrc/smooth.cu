@@ -103,7 +103,7 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
         for (int t = 0; t < n_stream; ++t) {
             const int ks = p.sweeps / n_stream + (t < p.sweeps % n_stream ? 1 : 0);
             if constexpr (sizeof(T) == 4)
-                LAUNCH(kind, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, run, s));
+                LAUNCH(kind, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, s));
             else
                 LAUNCH(kind, 1, launch_ras_stream64(g, k, omega, ks, ax, ay, bx, by, s));
             ++passes;

@@ -50,21 +50,9 @@ namespace {
 constexpr int ST_COLS = 128;     // columns of a strip
 constexpr int ST_PAIRS = 4;      // strips (pairs of warps) per CTA
 constexpr int ST_THREADS = ST_PAIRS * 64;
-constexpr int ST_FIELDS = 8;     // vx, vy, eta_c, eta_n, bx, by, 1/dx, 1/dy
 constexpr int ST_ROW = ST_FIELDS * ST_COLS;           // elements of a staged row
 constexpr int ST_MIN_SWEEPS = 3, ST_MAX_SWEEPS = 8;   // sweeps of a pass
 constexpr long long ST_MIN_CELLS = 600000;            // smallest grid
-
-struct StreamArgs {
-    GridDesc<float> g;
-    const float *f[ST_FIELDS];
-    float omega;
-    float *ox, *oy;
-    int sweeps;       // 2 KL or 2 KL - 1
-    int strips, segs; // column strips and row segments: one pair of warps each
-    int rows;         // cell rows per segment
-    int hl, own;      // columns left of the owned ones, and owned columns, of a strip
-};
 
 // 16-byte asynchronous copy of `bytes` (0 to 16) source bytes, the rest zero
 __device__ __forceinline__ void cp_async16z(uint32_t dst, const float *src, int bytes)
@@ -131,22 +119,39 @@ struct StreamShape {
     static_assert(D % N == 0, "slots repeat with the unrolled steps");
 };
 
-// `a.sweeps` = 2 KL - ODD sweeps of one strip and segment per pair of warps.
-// SQ: square cells (one coefficient for Txx and Tyy, one scaled shear), as in the pair
+// 2 KL - ODD sweeps of one strip and segment per pair of warps.  BATCH: of the
+// tasks of a table of grids, else of the grid `one`.  SQ: square cells (one coefficient for Txx and Tyy, one scaled shear), as in the pair
 // kernel.
-template <int KL, bool ODD, bool SQ>
-__global__ void __launch_bounds__(ST_THREADS, 1) k_ras_stream(const __grid_constant__ StreamArgs a)
+template <int KL, bool ODD, bool SQ, bool BATCH>
+__global__ void __launch_bounds__(ST_THREADS, 1)
+    k_ras_stream(const __grid_constant__ StreamEntry one, const StreamEntry *__restrict__ tab,
+                 const StreamTask *__restrict__ tasks, int ntasks, const int *__restrict__ live)
 {
     using Sh = StreamShape<KL>;
     constexpr int N = Sh::N, D = Sh::D, PF = Sh::PF;
     extern __shared__ __align__(16) float smem[];
+    __shared__ StreamEntry held[BATCH ? ST_PAIRS : 1];
     // (the shuffle tells the compiler that the warp number is uniform)
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = (int)threadIdx.x & 31;
     const int pair = warp % ST_PAIRS; // each SM partition holds a front and a back warp
     const bool back = warp >= ST_PAIRS;
     const int id = (int)blockIdx.x * ST_PAIRS + pair;
-    if (id >= a.strips * a.segs) return; // both warps of a pair; pairs never meet
-    const int strip = id % a.strips, seg = id / a.strips;
+    if (id >= ntasks) return; // both warps of a pair; pairs never meet
+    int piece = id;
+    if (BATCH) {
+        const StreamTask t = tasks[id];
+        if (live && !live[tab[t.entry].inst]) return;
+        piece = t.part;
+        if (!back) {
+            constexpr int W = (int)(sizeof(StreamEntry) / 4);
+            static_assert(sizeof(StreamEntry) % 4 == 0, "copied by words");
+            for (int w = lane; w < W; w += 32)
+                reinterpret_cast<int *>(&held[BATCH ? pair : 0])[w] = reinterpret_cast<const int *>(&tab[t.entry])[w];
+        }
+        pair_sync(pair);
+    }
+    const StreamEntry &a = BATCH ? held[BATCH ? pair : 0] : one;
+    const int strip = piece % a.strips, seg = piece / a.strips;
     const int nx = a.g.nx, ny = a.g.ny, n = a.sweeps;
     const int c0 = strip * a.own - a.hl + 4 * lane; // first of this lane's columns (a multiple of four, may lie outside)
     const int y0 = seg * a.rows, y1 = min(y0 + a.rows, ny);
@@ -292,30 +297,61 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_ras_stream(const __grid_const
     cp_wait<0>(); // no copy outlives the warp
 }
 
-template <int KL>
-void (*pick_stream(bool odd, bool square))(StreamArgs)
+using StreamKernel = void (*)(StreamEntry, const StreamEntry *, const StreamTask *, int, const int *);
+
+template <int KL, bool BATCH>
+StreamKernel pick_stream(bool odd, bool square)
 {
-    if (odd) return square ? k_ras_stream<KL, true, true> : k_ras_stream<KL, true, false>;
-    return square ? k_ras_stream<KL, false, true> : k_ras_stream<KL, false, false>;
+    if (odd) return square ? k_ras_stream<KL, true, true, BATCH> : k_ras_stream<KL, true, false, BATCH>;
+    return square ? k_ras_stream<KL, false, true, BATCH> : k_ras_stream<KL, false, false, BATCH>;
+}
+
+template <bool BATCH>
+cudaError_t run(int sweeps, bool square, const StreamEntry &one, const StreamEntry *tab, const StreamTask *tasks,
+                int ntasks, const int *live, cudaStream_t s)
+{
+    const int kl = (sweeps + 1) / 2;
+    const bool odd = sweeps & 1;
+    const StreamKernel kern = kl == 2   ? pick_stream<2, BATCH>(odd, square)
+                              : kl == 3 ? pick_stream<3, BATCH>(odd, square)
+                                        : pick_stream<4, BATCH>(odd, square);
+    const int elems = kl == 2 ? StreamShape<2>::SMEM : kl == 3 ? StreamShape<3>::SMEM : StreamShape<4>::SMEM;
+    const size_t smem = (size_t)ST_PAIRS * elems * sizeof(float);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(ntasks + ST_PAIRS - 1) / ST_PAIRS, ST_THREADS, smem, s>>>(one, tab, tasks, ntasks, live);
+    return cudaGetLastError();
+}
+
+int stream_wave()
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(sms, 1) * ST_PAIRS;
 }
 
 } // namespace
 
 int stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run)
 {
+    return stream_batch_passes((long long)g.nx * g.ny, sweeps, run);
+}
+
+int stream_batch_passes(long long cells, int sweeps, const RasRun &run)
+{
     if (!run.allow_tma || run.pair_mode != 1 || sweeps < ST_MIN_SWEEPS) return 0;
     // Below this a segment's 2 n extra rows outweigh the tiles' halo: 40 sweeps
     // take 101 us either way at 768^2, 80 (48 x 64 tiles: 70) at 512^2 and 111
     // (132) at 1024^2.
-    if ((long long)g.nx * g.ny < ST_MIN_CELLS) return 0;
+    if (cells < ST_MIN_CELLS) return 0;
     return (sweeps + ST_MAX_SWEEPS - 1) / ST_MAX_SWEEPS;
 }
 
-cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
-                              const float *vx, const float *vy, float *ox, float *oy, const RasRun &run, cudaStream_t s)
+StreamEntry stream_entry(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps, const float *vx,
+                         const float *vy, float *ox, float *oy)
 {
-    if (!c.inv_dx || !c.inv_dy || sweeps < ST_MIN_SWEEPS || sweeps > ST_MAX_SWEEPS) return cudaErrorInvalidValue;
-    StreamArgs a;
+    StreamEntry a{};
     a.g = g;
     a.omega = omega;
     a.ox = ox;
@@ -328,22 +364,58 @@ cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, 
     a.hl = sweeps <= 4 ? 4 : 8;
     a.own = ST_COLS - 2 * a.hl;
     a.strips = (g.nx + a.own - 1) / a.own;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int kl = (sweeps + 1) / 2;
-    const int segs = std::max(1, sms * ST_PAIRS / a.strips); // one wave of pairs
-    a.rows = (g.ny + segs - 1) / segs;
-    a.segs = (g.ny + a.rows - 1) / a.rows;
-    const bool sq = g.square != 0, odd = sweeps & 1;
-    void (*const kern)(StreamArgs) =
-        kl == 2 ? pick_stream<2>(odd, sq) : kl == 3 ? pick_stream<3>(odd, sq) : pick_stream<4>(odd, sq);
-    const int elems = kl == 2 ? StreamShape<2>::SMEM : kl == 3 ? StreamShape<3>::SMEM : StreamShape<4>::SMEM;
-    const size_t smem = (size_t)ST_PAIRS * elems * sizeof(float);
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<(a.strips * a.segs + ST_PAIRS - 1) / ST_PAIRS, ST_THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return a;
+}
+
+int stream_split(StreamEntry *e, int n)
+{
+    // the strips' rows, and the shortest segment that keeps the tasks within
+    // one wave (several where a wave's share is long: finer pieces even out
+    // grids of different heights, at 2 n + 1 extra rows each)
+    long long total = 0;
+    int longest = 1;
+    for (int q = 0; q < n; ++q) {
+        total += (long long)e[q].strips * e[q].g.ny;
+        longest = std::max(longest, e[q].g.ny);
+    }
+    const long long wave = stream_wave(), share = total / wave;
+    const long long want = wave * (n == 1 ? 1 : std::max(1LL, std::min(8LL, share / 100)));
+    auto tasks = [&](int rows) {
+        long long t = 0;
+        for (int q = 0; q < n; ++q) t += (long long)e[q].strips * ((e[q].g.ny + rows - 1) / rows);
+        return t;
+    };
+    int lo = 1, hi = longest; // tasks(hi) may exceed `want` (many strips): then one segment each
+    while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        if (tasks(mid) <= want) hi = mid;
+        else lo = mid + 1;
+    }
+    int t = 0;
+    for (int q = 0; q < n; ++q) {
+        const int segs = (e[q].g.ny + lo - 1) / lo;
+        e[q].rows = (e[q].g.ny + segs - 1) / segs;
+        e[q].segs = (e[q].g.ny + e[q].rows - 1) / e[q].rows;
+        t += e[q].strips * e[q].segs;
+    }
+    return t;
+}
+
+cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
+                              const float *vx, const float *vy, float *ox, float *oy, cudaStream_t s)
+{
+    if (!c.inv_dx || !c.inv_dy || sweeps < ST_MIN_SWEEPS || sweeps > ST_MAX_SWEEPS) return cudaErrorInvalidValue;
+    StreamEntry a = stream_entry(g, c, omega, sweeps, vx, vy, ox, oy);
+    const int ntasks = stream_split(&a, 1);
+    return run<false>(sweeps, g.square != 0, a, nullptr, nullptr, ntasks, nullptr, s);
+}
+
+cudaError_t launch_ras_stream_batch(const StreamEntry *tab, const StreamTask *tasks, int ntasks, int sweeps,
+                                    bool square, const int *live, cudaStream_t s)
+{
+    if (sweeps < ST_MIN_SWEEPS || sweeps > ST_MAX_SWEEPS) return cudaErrorInvalidValue;
+    if (ntasks <= 0) return cudaSuccess;
+    return run<true>(sweeps, square, StreamEntry{}, tab, tasks, ntasks, live, s);
 }
 
 } // namespace stokes

@@ -102,6 +102,30 @@ def test_batched_smoothing_is_bitwise_the_single_context(api, dtype, kw, tma):
     b.close()
 
 
+@pytest.mark.parametrize("kw", [dict(variant="ras", sweeps=17, tile=(48, 64), k=8, overlap=7, seed=3),
+                                dict(variant="fused", sweeps=6), dict(variant="ras", sweeps=3, tile=(32, 32), k=2,
+                                                                      overlap=1, seed=4)])
+def test_batched_row_streaming_is_the_global_jacobi(api, kw):
+    """Large FP32 batches with o >= k - 1 stream the rows of all instances in one
+    launch a pass: grids of very different widths and heights, square and
+    oblong cells, odd and even pass counts, value for value separate-pass Jacobi
+    on a context each."""
+    probs = problems([(900, 500), (64, 64), (113, 700), (3, 5), (250, 300), (1000, 120)], 30)
+    wide = inputs.sinker_problem(224, 224, eta_in=1e3, lx=1.0, ly=0.6)
+    wide.eta_c, wide.eta_n = inputs.random_viscosity(224, 224, 77, (-2.0, 2.0))
+    probs.append(wide)
+    v0 = [inputs.random_velocity(q.nx, q.ny, 300 + i) for i, q in enumerate(probs)]
+    p = [inputs.random_pressure(q.nx, q.ny, 400 + i, 0.5) for i, q in enumerate(probs)]
+    ref = single_results(api, probs, "f32", v0, p,
+                         lambda c, vx, vy, pt: c.smooth(vx, vy, pt, variant="jacobi", sweeps=kw["sweeps"]))
+    b = batch_context(api, probs, "f32")
+    vx, vy = b.pack([v[0] for v in v0], "vx"), b.pack([v[1] for v in v0], "vy")
+    b.smooth(vx, vy, b.pack(p, "p"), **kw)
+    for i in range(len(probs)):
+        assert np.array_equal(b.unpack(vx, "vx", i), ref[i][0]) and np.array_equal(b.unpack(vy, "vy", i), ref[i][1]), i
+    b.close()
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 def test_batched_energy_matches_the_single_context(api, dtype):
     probs = problems(SIZES, 20)
