@@ -175,6 +175,12 @@ int stream_batch_passes(long long cells, int sweeps, const RasRun &run);
 // and square or not; entries whose live[inst] is 0 are skipped.
 cudaError_t launch_ras_stream_batch(const StreamEntry *tab, const StreamTask *tasks, int ntasks, int sweeps,
                                     bool square, const int *live, cudaStream_t s);
+// Red-black Gauss-Seidel by row streaming (FP32, rbgs_kernels.cu): the passes
+// that `sweeps` sweeps take, 0 where launch_rbgs_sweep runs them instead, and
+// one pass of one or two sweeps.
+int rbgs_stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run);
+cudaError_t launch_rbgs_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
+                               const float *vx, const float *vy, float *ox, float *oy, cudaStream_t s);
 // All sweeps of a small grid's damped Jacobi in one launch, in place
 // (cluster_kernels.cu): whether a smoothing of `sweeps` sweeps takes it, and
 // the launch.

@@ -20,14 +20,16 @@ bool takes_cluster(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
     return any_traversal(p) && cluster_takes<T>(g.nx, g.ny, p.sweeps, run);
 }
 
-// passes of the row-streaming kernel for this smoothing, 0 if it does not take
-// it: a RAS schedule with overlap >= k - 1 is global Jacobi in any traversal,
-// and fused Jacobi's sweeps need not each cross the grid before the next
-// begins (20 sweeps of 4001 x 2999: 408 us, 1822 us as 20 passes of
-// k_jacobi_rows).  Separate-pass and blocked Jacobi keep their own passes.
+// passes of a row-streaming kernel for this smoothing, 0 if none takes it: red-
+// black Gauss-Seidel's own; else a RAS schedule with overlap >= k - 1 is global
+// Jacobi in any traversal, and fused Jacobi's sweeps need not each cross the
+// grid before the next begins (20 sweeps of 4001 x 2999: 408 us, 1822 us as 20
+// passes of k_jacobi_rows).  Separate-pass and blocked Jacobi keep their passes.
 template <typename T>
 int stream_passes_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
 {
+    if constexpr (sizeof(T) == 4)
+        if (p.variant == STOKES_RBGS) return rbgs_stream_passes(g, p.sweeps, run);
     if (!any_traversal(p)) return 0;
     if constexpr (sizeof(T) == 4) return stream_passes(g, p.sweeps, run);
     else return stream64_passes(g, p.sweeps, run);
@@ -63,7 +65,9 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + p.k - 1) / p.k : 0;
     const bool cluster = takes_cluster(g, p, run);
     const int n_stream = stream_passes_of(g, p, run);
-    const int kind = p.variant == STOKES_RAS ? STOKES_K_RAS : STOKES_K_JACOBI;
+    const int kind = p.variant == STOKES_RAS    ? STOKES_K_RAS
+                     : p.variant == STOKES_RBGS ? STOKES_K_RBGS
+                                                : STOKES_K_JACOBI;
     if ((cluster || n_stream > 0) && p.variant == STOKES_RAS && p.shift_mode == STOKES_SHIFT_LIST)
         for (int t = 0; t < n_outer; ++t) // the shifts change nothing, but bad ones stay refused
             if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 || p.shifts[2 * t + 1] >= p.tj)
@@ -102,10 +106,13 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     if (n_stream > 0) {
         for (int t = 0; t < n_stream; ++t) {
             const int ks = p.sweeps / n_stream + (t < p.sweeps % n_stream ? 1 : 0);
-            if constexpr (sizeof(T) == 4)
-                LAUNCH(kind, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, s));
-            else
+            if constexpr (sizeof(T) == 8) {
                 LAUNCH(kind, 1, launch_ras_stream64(g, k, omega, ks, ax, ay, bx, by, s));
+            } else if (p.variant == STOKES_RBGS) {
+                LAUNCH(kind, 1, launch_rbgs_stream(g, k, omega, ks, ax, ay, bx, by, s));
+            } else {
+                LAUNCH(kind, 1, launch_ras_stream(g, k, omega, ks, ax, ay, bx, by, s));
+            }
             ++passes;
             advance();
         }

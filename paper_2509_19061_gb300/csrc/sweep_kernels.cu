@@ -16,7 +16,8 @@
 // fly (two fewer fields to read; the kernel is memory-bound); FP64 reads the
 // precomputed 1/diag arrays (an FP64 reciprocal costs more than the bytes).
 //
-// Red-black Gauss-Seidel (k_rbgs_tile).  One launch runs a whole sweep, the
+// Red-black Gauss-Seidel (k_rbgs_tile; large FP32 grids stream by rows,
+// rbgs_kernels.cu).  One launch runs a whole sweep, the
 // four half-sweeps vx-red, vx-black, vy-red, vy-black, on a tile grown by a
 // halo: a half-sweep's points depend on the previous half-sweeps only
 // within one cell, so vx-red runs on the tile grown by 3 cells, vx-black by

@@ -759,6 +759,31 @@ def test_row_streaming_f64_equals_global_jacobi(api, nx, ny, sweeps, square):
         assert np.array_equal(outs[0][0], outs[-1][0]) and np.array_equal(outs[0][1], outs[-1][1])
 
 
+@pytest.mark.parametrize("nx,ny,sweeps,square", [
+    (1121, 400, 1, True), (1120, 401, 2, False), (896, 500, 3, True), (960, 450, 4, False), (113, 4000, 5, True),
+    (3, 140000, 2, False), (140000, 3, 3, True),
+])
+def test_rbgs_streaming_equals_the_tile_kernel(api, nx, ny, sweeps, square):
+    """Red-black Gauss-Seidel by row streaming (large FP32 grids): strips of
+    112 or 120 columns that end on, before and after the grid's edge, one and
+    two sweeps a pass, odd and even pass counts, with a pressure, moving walls
+    and NaN in the padding: value for value the tile kernel's."""
+    prob = rand_problem(nx, ny, 91, lx=1.0, ly=ny / nx if square else 0.7)
+    vx, vy = inputs.random_velocity(nx, ny, 92, 0.1)
+    vx[:, 0], vx[:, nx], vy[0], vy[ny] = 0.3, -0.2, 0.1, 0.4
+    p = inputs.random_pressure(nx, ny, 93)
+    outs = []
+    for pair in (0, 1):
+        r = Run(api, prob, "f32", (vx, vy), p)
+        r.ctx.set_option(api.STOKES_OPT_PAIRED, pair)
+        r.vx, r.vy = _with_canaries(api, r.ctx, r.vx, "vx"), _with_canaries(api, r.ctx, r.vy, "vy")
+        r.smooth(variant="rbgs", sweeps=sweeps)
+        outs.append(r.v())
+        assert np.isnan(r.vx.cpu().numpy()[ny:]).all()
+        r.ctx.close()
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("kw", [
     dict(variant="jacobi", sweeps=3), dict(variant="fused", sweeps=3), dict(variant="rbgs", sweeps=2),
