@@ -262,6 +262,25 @@ def test_ras3d_column_kernel_fp32_energy_error(api, o3, tile, k, o):
     assert err <= FP32_ENERGY_TOL
 
 
+@pytest.mark.parametrize("dtype,tile,k,o", [("f64", (30, 6, 6), 4, 0), ("f64", (28, 4, 4), 3, 1),
+                                            ("f32", (30, 6, 6), 4, 0), ("f32", (30, 10, 6), 3, 0),
+                                            ("f32", (30, 14, 6), 3, 0), ("f32", (28, 4, 8), 3, 1),
+                                            ("f32", (28, 8, 8), 3, 1)])
+def test_ras3d_column_kernel_cubic_cells(api, o3, dtype, tile, k, o):
+    """Cubic cells (hx = hy = hz) take the column kernel's form with one flux
+    coefficient and shears scaled where they are formed, in every window shape."""
+    nx, ny, nz = 64, 32, 16
+    prob = problem(nx, ny, nz, 41, (2.0, 1.0, 0.5))
+    cast = f32 if dtype == "f32" else (lambda a: a)
+    v0 = inputs.random_velocity3d(nx, ny, nz, 42, 0.1)
+    g = ogrid(o3, prob, cast)
+    b = o3.rhs(g, cast(prob.fx), cast(prob.fy), cast(prob.fz), None)
+    r = Run3(api, prob, dtype, v0)
+    r.smooth(variant="ras", sweeps=2 * k - 1, tile=tile, k=k, overlap=o, seed=5)
+    ref = o3.ras(g, b, 0.3, 2 * k - 1, tile, k, o, shift_mode=1, seed=5, v=tuple(cast(a) for a in v0))
+    assert rel(r.get(), ref) <= (F64_TOL if dtype == "f64" else FP32_ENERGY_TOL)
+
+
 @pytest.mark.parametrize("variant,kw", [("fused", {}), ("ras", dict(tile=(8, 8, 8), k=2, overlap=1)),
                                         ("ras", dict(tile=(8, 8, 4), k=4, overlap=0))])
 def test_fp32_energy_error_3d(api, o3, variant, kw):
