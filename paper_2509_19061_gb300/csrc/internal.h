@@ -304,10 +304,12 @@ struct SmoothSpec {
 // caller then treats (sx, sy) as the velocity and (vx, vy) as the scratch.
 // With a second scratch pair (tx, ty) (and no `swapped`), an odd number of
 // passes ends in (vx, vy) by alternating between the two scratch pairs.
+// `zero_walls`: the walls of (vx, vy) and of the scratch pair are zero already
+// (the levels of a V-cycle), so none are copied.
 template <typename T>
 int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx, T *sy, const SmoothSpec &p,
                    const RasRun &run, cudaStream_t s, LaunchHook &hook, bool *swapped = nullptr, T *tx = nullptr,
-                   T *ty = nullptr);
+                   T *ty = nullptr, bool zero_walls = false);
 // ping-pong passes of one smoothing call
 template <typename T>
 int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run);

@@ -51,7 +51,8 @@ int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
 
 template <typename T>
 int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx, T *sy, const SmoothSpec &p,
-                   const RasRun &run, cudaStream_t s, LaunchHook &hook, bool *swapped, T *tx, T *ty)
+                   const RasRun &run, cudaStream_t s, LaunchHook &hook, bool *swapped, T *tx, T *ty,
+                   bool zero_walls)
 {
     if (swapped) *swapped = false;
     const T omega = (T)p.omega;
@@ -84,7 +85,7 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     const int n_pass = smooth_passes(g, p, run);
     const bool three = tx && ty && !swapped && n_pass >= 3 && (n_pass & 1);
     T *ax = vx, *ay = vy, *bx = sx, *by = sy;
-    LAUNCH(STOKES_K_COPY, 1, launch_copy_walls<T>(g, vx, vy, sx, sy, s));
+    if (!zero_walls) LAUNCH(STOKES_K_COPY, 1, launch_copy_walls<T>(g, vx, vy, sx, sy, s));
     if (three) LAUNCH(STOKES_K_COPY, 1, launch_copy_walls<T>(g, vx, vy, tx, ty, s));
     int passes = 0;
     // after pass `passes` (1-based) wrote (bx, by): the source and target of the next
@@ -162,9 +163,9 @@ template int smooth_passes<float>(const GridDesc<float> &, const SmoothSpec &, c
 template int smooth_passes<double>(const GridDesc<double> &, const SmoothSpec &, const RasRun &);
 template int smooth_buffers<float>(const GridDesc<float> &, const Coeffs<float> &, float *, float *, float *,
                                    float *, const SmoothSpec &, const RasRun &, cudaStream_t, LaunchHook &, bool *,
-                                   float *, float *);
+                                   float *, float *, bool);
 template int smooth_buffers<double>(const GridDesc<double> &, const Coeffs<double> &, double *, double *, double *,
                                     double *, const SmoothSpec &, const RasRun &, cudaStream_t, LaunchHook &, bool *,
-                                    double *, double *);
+                                    double *, double *, bool);
 
 } // namespace stokes
