@@ -138,13 +138,15 @@ __global__ void __launch_bounds__(RD_THREADS) k_dot_z(int nx, int ny, int pitch,
     block_store2(s0, 0.0, partials);
 }
 
-// p = (T) z + beta p at the unknowns, z in its own precision; FIRST: p = (T) z
+// p = (T) z + beta p at the unknowns, z in its own precision, beta = -<z, q> /
+// <p, q> from the device scalars *zq and *pq; FIRST: p = (T) z
 template <typename T, typename Tz, bool FIRST>
-__global__ void __launch_bounds__(RD_THREADS) k_direction_z(int nx, int ny, int pitch, double beta,
+__global__ void __launch_bounds__(RD_THREADS) k_direction_z(int nx, int ny, int pitch, const double *__restrict__ zq,
+                                                            const double *__restrict__ pq,
                                                             const Tz *__restrict__ zx, const Tz *__restrict__ zy,
                                                             T *__restrict__ px, T *__restrict__ py)
 {
-    const T bt = (T)beta;
+    const T bt = FIRST ? T(0) : (T)(-*zq / *pq);
     for_unknowns(nx, ny, pitch, [&](size_t q, int comp) {
         T *p = comp ? py : px;
         const T z = (T)(comp ? zy : zx)[q];
@@ -152,9 +154,11 @@ __global__ void __launch_bounds__(RD_THREADS) k_direction_z(int nx, int ny, int 
     });
 }
 
-// v += a p, r -= a q, bi = (Ti) r; returns (sum r_new^2 w, 0)
+// v += a p, r -= a q, bi = (Ti) r with a = <p, r> / <p, q> from the device pair
+// pqr = (<p, q>, <p, r>); returns (sum r_new^2 w, 0)
 template <typename T, typename Ti>
-__global__ void __launch_bounds__(RD_THREADS) k_cg_update_cast(int nx, int ny, int pitch, double a,
+__global__ void __launch_bounds__(RD_THREADS) k_cg_update_cast(int nx, int ny, int pitch,
+                                                               const double *__restrict__ pqr,
                                                                const T *__restrict__ px, const T *__restrict__ py,
                                                                const T *__restrict__ qx, const T *__restrict__ qy,
                                                                T *__restrict__ vx, T *__restrict__ vy,
@@ -163,7 +167,7 @@ __global__ void __launch_bounds__(RD_THREADS) k_cg_update_cast(int nx, int ny, i
                                                                Ti *__restrict__ bix, Ti *__restrict__ biy,
                                                                double *__restrict__ partials)
 {
-    const T at = (T)a;
+    const T at = (T)(pqr[1] / pqr[0]);
     double s0 = 0.0;
     for_unknowns(nx, ny, pitch, [&](size_t q, int comp) {
         T *v = comp ? vy : vx;
@@ -315,21 +319,21 @@ cudaError_t kry_dot_z(const KrylovView &k, const Tz *zx, const Tz *zy, const T *
 }
 
 template <typename T, typename Tz>
-cudaError_t kry_direction_z(const KrylovView &k, double beta, const Tz *zx, const Tz *zy, T *px, T *py,
-                            cudaStream_t s)
+cudaError_t kry_direction_z(const KrylovView &k, const double *zq, const double *pq, const Tz *zx, const Tz *zy,
+                            T *px, T *py, cudaStream_t s)
 {
-    if (beta == 0.0)
-        k_direction_z<T, Tz, true><<<RD_BLOCKS, RD_THREADS, 0, s>>>(k.nx, k.ny, k.pitch, beta, zx, zy, px, py);
+    if (!zq)
+        k_direction_z<T, Tz, true><<<RD_BLOCKS, RD_THREADS, 0, s>>>(k.nx, k.ny, k.pitch, zq, pq, zx, zy, px, py);
     else
-        k_direction_z<T, Tz, false><<<RD_BLOCKS, RD_THREADS, 0, s>>>(k.nx, k.ny, k.pitch, beta, zx, zy, px, py);
+        k_direction_z<T, Tz, false><<<RD_BLOCKS, RD_THREADS, 0, s>>>(k.nx, k.ny, k.pitch, zq, pq, zx, zy, px, py);
     return cudaGetLastError();
 }
 
 template <typename T, typename Ti>
-cudaError_t kry_update_cast(const KrylovView &k, double a, const T *px, const T *py, const T *qx, const T *qy, T *vx,
-                            T *vy, T *rx, T *ry, const T *ix, const T *iy, Ti *bix, Ti *biy, cudaStream_t s)
+cudaError_t kry_update_cast(const KrylovView &k, const double *pqr, const T *px, const T *py, const T *qx,
+                            const T *qy, T *vx, T *vy, T *rx, T *ry, const T *ix, const T *iy, Ti *bix, Ti *biy, cudaStream_t s)
 {
-    k_cg_update_cast<T, Ti><<<RD_BLOCKS, RD_THREADS, 0, s>>>(k.nx, k.ny, k.pitch, a, px, py, qx, qy, vx, vy, rx, ry,
+    k_cg_update_cast<T, Ti><<<RD_BLOCKS, RD_THREADS, 0, s>>>(k.nx, k.ny, k.pitch, pqr, px, py, qx, qy, vx, vy, rx, ry,
                                                              ix, iy, bix, biy, k.partials);
     k_final2<<<1, 64, 0, s>>>(k.partials, RD_BLOCKS, k.out);
     return cudaGetLastError();
@@ -338,10 +342,10 @@ cudaError_t kry_update_cast(const KrylovView &k, double a, const T *px, const T 
 #define INST_Z(T, Tz)                                                                                              \
     template cudaError_t kry_dot_z<T, Tz>(const KrylovView &, const Tz *, const Tz *, const T *, const T *,       \
                                           cudaStream_t);                                                           \
-    template cudaError_t kry_direction_z<T, Tz>(const KrylovView &, double, const Tz *, const Tz *, T *, T *,     \
-                                                cudaStream_t);                                                     \
-    template cudaError_t kry_update_cast<T, Tz>(const KrylovView &, double, const T *, const T *, const T *,       \
-                                                const T *, T *, T *, T *, T *, const T *, const T *, Tz *, Tz *,  \
+    template cudaError_t kry_direction_z<T, Tz>(const KrylovView &, const double *, const double *, const Tz *,    \
+                                                const Tz *, T *, T *, cudaStream_t);                               \
+    template cudaError_t kry_update_cast<T, Tz>(const KrylovView &, const double *, const T *, const T *,          \
+                                                const T *, const T *, T *, T *, T *, T *, const T *, const T *, Tz *, Tz *,  \
                                                 cudaStream_t);
 INST_Z(double, float)
 INST_Z(double, double)

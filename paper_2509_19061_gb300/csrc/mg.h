@@ -72,12 +72,12 @@ cudaError_t kry_dot2(const KrylovView &k, const T *ax, const T *ay, const T *bx,
                      const T *cy, cudaStream_t s);
 template <typename T, typename Tz> // (<z, b>, 0) with z in its own precision
 cudaError_t kry_dot_z(const KrylovView &k, const Tz *zx, const Tz *zy, const T *bx, const T *by, cudaStream_t s);
-template <typename T, typename Tz> // p = (T) z + beta p (beta = 0: p = (T) z)
-cudaError_t kry_direction_z(const KrylovView &k, double beta, const Tz *zx, const Tz *zy, T *px, T *py,
-                            cudaStream_t s);
-template <typename T, typename Ti> // kry_update, and bi = (Ti) r_new at the unknowns
-cudaError_t kry_update_cast(const KrylovView &k, double a, const T *px, const T *py, const T *qx, const T *qy, T *vx,
-                            T *vy, T *rx, T *ry, const T *ix, const T *iy, Ti *bix, Ti *biy, cudaStream_t s);
+template <typename T, typename Tz> // p = (T) z - (*zq / *pq) p, device scalars (zq = NULL: p = (T) z)
+cudaError_t kry_direction_z(const KrylovView &k, const double *zq, const double *pq, const Tz *zx, const Tz *zy,
+                            T *px, T *py, cudaStream_t s);
+template <typename T, typename Ti> // kry_update with a = pqr[1] / pqr[0] (device), and bi = (Ti) r_new at the unknowns
+cudaError_t kry_update_cast(const KrylovView &k, const double *pqr, const T *px, const T *py, const T *qx,
+                            const T *qy, T *vx, T *vy, T *rx, T *ry, const T *ix, const T *iy, Ti *bix, Ti *biy, cudaStream_t s);
 template <typename T> // q = M p (library eta_n: boundary nodes zero); out = (<p, q>, <p, r>);
                       // ax, ay: coefficients from kry_coef, or NULL to form them per flux
 cudaError_t kry_apply_dot(const KrylovView &k, const GridDesc<T> &g, const T *ec, const T *en, const T *ax,
