@@ -104,7 +104,7 @@ template <typename T>
 cudaError_t launch_energy_raw(const GridDesc<T> &g, const T *eta_c, const T *eta_n, const T *fx, const T *fy,
                               const T *p, const T *vx, const T *vy, double *partials, double *out, cudaStream_t s);
 
-// ---- FP64 operator by row-marching warps (op_rows.cu) ---------------------
+// ---- the operator by row-marching warps (op_rows.cu) ----------------------
 // Whether a grid is large enough for it; every buffer it gets starts on a
 // 16-byte boundary.
 bool op_rows_takes(int nx, int ny);
@@ -115,6 +115,10 @@ cudaError_t op_rows_apply(const GridDesc<double> &g, const double *ec, const dou
 cudaError_t op_rows_residual(const GridDesc<double> &g, const double *ec, const double *en, const double *bx,
                              const double *by, const double *vx, const double *vy, double *rx, double *ry,
                              cudaStream_t s);
+// coarse b = P^T (b - M v) / 4 of the next coarser level (pitch cpitch), zero off its unknowns
+template <typename T>
+cudaError_t op_rows_restrict(const GridDesc<T> &g, const T *ec, const T *en, const T *bx, const T *by, const T *vx,
+                             const T *vy, T *cbx, T *cby, int cpitch, cudaStream_t s);
 // ---- tiled / RAS kernel (ras_kernels.cu) ---------------------------------
 struct TileGrid {
     int ti, tj;   // tile size (cells)

@@ -64,9 +64,10 @@ int alloc_level(MgLevel &l, int nx, int ny, double hx, double hy, size_t es, boo
     l.hy = hy;
     l.pitch = ((nx + 1) + 31) / 32 * 32;
     l.elems = (size_t)(ny + 1) * (size_t)l.pitch;
-    void **fs[] = {&l.ec, &l.en, &l.bx, &l.by, &l.rx, &l.ry, &l.sx, &l.sy, &l.ivx, &l.ivy};
-    const int nf = inv ? 10 : 8;
-    for (int f = 0; f < nf; ++f) {
+    void **fs[] = {&l.ec, &l.en, &l.bx, &l.by, &l.sx, &l.sy, &l.rx, &l.ry, &l.ivx, &l.ivy};
+    const bool resid = es == 8 && !mg_restrict_fused<double>(nx, ny);
+    for (int f = 0; f < 10; ++f) {
+        if (f >= 6 && !(f < 8 ? resid : inv)) continue;
         cudaError_t e = cudaMalloc(fs[f], l.elems * es);
         if (e == cudaSuccess) e = cudaMemsetAsync(*fs[f], 0, l.elems * es, s);
         if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? STOKES_ERR_OOM : STOKES_ERR_CUDA;
@@ -276,8 +277,8 @@ int enqueue_precond(MgHierarchy *h, const Tc *rx, const Tc *ry, Tc *zx, Tc *zy, 
         MgLevel &f = h->lv[l];
         st = smooth_level(f, l, 0);
         if (st != STOKES_OK) return st;
-        LAUNCH(STOKES_K_MG, 1, mg_residual<Ti>(f, s));
-        LAUNCH(STOKES_K_MG, 1, mg_restrict<Ti>(f, h->lv[l + 1], s));
+        LAUNCH(STOKES_K_MG, mg_restrict_fused<Ti>(f.nx, f.ny) ? 1 : 2,
+               mg_residual_restrict<Ti>(f, h->lv[l + 1], s));
     }
     // coarsest: exact solve
     LAUNCH(STOKES_K_MG, 3, mg_dense_solve<Ti>(h->lv[L - 1], h->n, h->Ainv, h->bvec, h->xvec, s));

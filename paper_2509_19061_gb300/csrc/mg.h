@@ -111,8 +111,14 @@ template <typename Ts, typename Td>
 cudaError_t mg_cast(size_t n, const void *src, void *dst, cudaStream_t s);
 template <typename T>
 cudaError_t mg_residual(const MgLevel &l, cudaStream_t s);
+// Whether a level's residual and its restriction are one launch, without l.rx and l.ry
 template <typename T>
-cudaError_t mg_restrict(const MgLevel &f, const MgLevel &c, cudaStream_t s);
+bool mg_restrict_fused(int nx, int ny)
+{
+    return sizeof(T) == 4 || op_rows_takes(nx, ny);
+}
+template <typename T> // c.b = P^T (f.b - M f.v) / 4
+cudaError_t mg_residual_restrict(const MgLevel &f, const MgLevel &c, cudaStream_t s);
 template <typename T>
 cudaError_t mg_prolong_add(const MgLevel &f, const MgLevel &c, cudaStream_t s);
 template <typename T>

@@ -422,8 +422,14 @@ cudaError_t mg_residual(const MgLevel &l, cudaStream_t s)
 }
 
 template <typename T>
-cudaError_t mg_restrict(const MgLevel &f, const MgLevel &c, cudaStream_t s)
+cudaError_t mg_residual_restrict(const MgLevel &f, const MgLevel &c, cudaStream_t s)
 {
+    if (mg_restrict_fused<T>(f.nx, f.ny))
+        return op_rows_restrict(make_grid<T>(f.nx, f.ny, f.pitch, f.hx, f.hy), (const T *)f.ec, (const T *)f.en,
+                                (const T *)f.bx, (const T *)f.by, (const T *)f.vx, (const T *)f.vy, (T *)c.bx,
+                                (T *)c.by, c.pitch, s);
+    const cudaError_t e = mg_residual<T>(f, s);
+    if (e != cudaSuccess) return e;
     k_restrict<T><<<grid2d(c.nx + 1, c.ny + 1), dim3(BX, BY), 0, s>>>(f.nx, f.ny, f.pitch, c.nx, c.ny, c.pitch,
                                                                        (const T *)f.rx, (const T *)f.ry, (T *)c.bx,
                                                                        (T *)c.by);
@@ -511,7 +517,7 @@ cudaError_t mg_dense_solve(const MgLevel &l, int n, const double *Ainv, double *
 #define INST(T)                                                                                                    \
     template cudaError_t mg_coarsen_eta<T>(const MgLevel &, const MgLevel &, cudaStream_t);                        \
     template cudaError_t mg_residual<T>(const MgLevel &, cudaStream_t);                                            \
-    template cudaError_t mg_restrict<T>(const MgLevel &, const MgLevel &, cudaStream_t);                           \
+    template cudaError_t mg_residual_restrict<T>(const MgLevel &, const MgLevel &, cudaStream_t);                  \
     template cudaError_t mg_prolong_add<T>(const MgLevel &, const MgLevel &, cudaStream_t);                        \
     template cudaError_t mg_dense_setup<T>(const MgLevel &, int, double *, double *, double *, int *,              \
                                            cudaStream_t);                                                          \

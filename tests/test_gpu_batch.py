@@ -231,6 +231,26 @@ def test_batched_defect_correction_is_bitwise_the_single_context(api, dtype, inn
     b.close()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_single_transfers_are_bitwise_the_batched_points(api, dtype):
+    """A single V-cycle forms the residual with its restriction by rows (levels
+    of FP64 from 100000 cells, of FP32 all); the batch takes a point at a time.  Levels whose columns end on, before and
+    after a strip of 60 (30 coarse), few and many rows, both cell shapes."""
+    import torch
+    probs = [inputs.sinker_problem(nx, ny, eta_in=1e2, lx=1.0, ly=r * ny / nx)
+             for nx, ny, r in ((120, 64, 1.0), (248, 32, 0.7), (56, 240, 1.0), (480, 256, 0.7), (352, 480, 1.0))]
+    v0 = [(np.zeros((q.ny, q.nx + 1)), np.zeros((q.ny + 1, q.nx))) for q in probs]
+    kw = dict(variant="jacobi", nu_max=2, inner=dtype, coarsest=4, krylov=False, tol=0.0, max_cycles=2)
+    ref = single_results(api, probs, dtype, v0, None, lambda c, vx, vy, pt: c.vcycle(vx, vy, pt, **kw))
+    for i, prob in enumerate(probs):
+        b = batch_context(api, [prob], dtype)
+        vx, vy = b.slab(), b.slab()
+        b.solve(vx, vy, None, **kw)
+        torch.cuda.synchronize()
+        assert np.array_equal(b.unpack(vx, "vx", 0), ref[i][0]) and np.array_equal(b.unpack(vy, "vy", 0), ref[i][1]), i
+        b.close()
+
+
 def test_batched_fcg_reaches_1e8_like_the_single_contexts(api):
     """Flexible CG to E_v <= 1e-8 on sinkers of uneven sizes and contrasts
     1e2..1e6 (the batched workload's recipe): every instance converges, in
