@@ -77,7 +77,8 @@ cudaError_t kry_direction_z(const KrylovView &k, const double *zq, const double 
                             T *px, T *py, cudaStream_t s);
 template <typename T, typename Ti> // kry_update with a = pqr[1] / pqr[0] (device), and bi = (Ti) r_new at the unknowns
 cudaError_t kry_update_cast(const KrylovView &k, const double *pqr, const T *px, const T *py, const T *qx,
-                            const T *qy, T *vx, T *vy, T *rx, T *ry, const T *ix, const T *iy, Ti *bix, Ti *biy, cudaStream_t s);
+                            const T *qy, T *vx, T *vy, T *rx, T *ry, const T *ix, const T *iy, Ti *bix, Ti *biy,
+                            cudaStream_t s);
 template <typename T> // q = M p (library eta_n: boundary nodes zero); out = (<p, q>, <p, r>);
                       // ax, ay: coefficients from kry_coef, or NULL to form them per flux
 cudaError_t kry_apply_dot(const KrylovView &k, const GridDesc<T> &g, const T *ec, const T *en, const T *ax,
