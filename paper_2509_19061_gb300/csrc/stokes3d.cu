@@ -1038,7 +1038,21 @@ int smooth_impl(stokes3d_ctx *c, T *vx, T *vy, T *vz, const T *p, const stokes3d
         k3_jacobi<T><<<gr, bl, 0, c->stream>>>(g, a, k, omega, B[0], B[1], B[2]);
         ++c->kernels;
     };
-    if (prm->variant == STOKES_JACOBI_FUSED) {
+    // A RAS schedule with overlap >= k - 1 is global Jacobi, and in 3D a box's
+    // halo costs more than k sweeps on chip save, so fused Jacobi runs it on
+    // large grids.  12 sweeps in FP32: 96^3 358 us fused, 360 to 473 by tiles
+    // with k = 2; 192^3 1777, 2160 to 3529; 320^3 6880, 9209 to 16796.  FP64: 47^3
+    // 498, 683 to 2544; 192^3 17.7 ms, 30 to 107.  (k = 1 keeps its tiles: 1823 us
+    // at 192^3 in FP32, but 12.4 ms for two sweeps of 320^3 in FP64, 13.3 fused.)
+    const bool exact = prm->variant == STOKES_RAS && prm->k >= 2 && prm->overlap >= prm->k - 1 &&
+                       (long long)c->nx * c->ny * c->nz >= (sizeof(T) == 4 ? 2000000 : 100000);
+    if (exact && prm->shift_mode == STOKES_SHIFT_LIST)
+        for (int t = 0; t < (prm->sweeps + prm->k - 1) / prm->k; ++t)
+            for (int d = 0; d < 3; ++d)
+                if (const int sh = prm->shifts[3 * t + d], e = d == 0 ? prm->tile_i : d == 1 ? prm->tile_j : prm->tile_k;
+                    sh < 0 || sh >= e)
+                    return STOKES_ERR_ARG;
+    if (prm->variant == STOKES_JACOBI_FUSED || exact) {
         for (int s = 0; s < prm->sweeps; ++s) {
             pass_jacobi();
             std::swap(A[0], B[0]);

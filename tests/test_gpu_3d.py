@@ -281,6 +281,24 @@ def test_ras3d_column_kernel_cubic_cells(api, o3, dtype, tile, k, o):
     assert rel(r.get(), ref) <= (F64_TOL if dtype == "f64" else FP32_ENERGY_TOL)
 
 
+@pytest.mark.parametrize("dtype,nx,ny,nz", [("f32", 161, 127, 101), ("f64", 61, 50, 40)])
+def test_ras3d_exact_schedules_on_large_grids(api, dtype, nx, ny, nz):
+    """overlap >= k - 1 on a large grid is run as fused Jacobi, odd and even
+    sweep counts, and still refuses a shift outside its tile."""
+    prob = problem(nx, ny, nz, 43)
+    v0 = inputs.random_velocity3d(nx, ny, nz, 44, 0.1)
+    for sweeps in (3, 4):
+        outs = []
+        for kw in (dict(variant="fused"), dict(variant="ras", tile=(8, 8, 8), k=2, overlap=1, seed=6)):
+            r = Run3(api, prob, dtype, v0)
+            r.smooth(sweeps=sweeps, **kw)
+            outs.append(r.get())
+        assert all(np.array_equal(x, y) for x, y in zip(*outs))
+    with pytest.raises(api.StokesError) as e:
+        r.smooth(variant="ras", sweeps=2, tile=(8, 8, 8), k=2, overlap=1, shifts=[[0, 8, 0]])
+    assert e.value.status == api.STOKES_ERR_ARG
+
+
 @pytest.mark.parametrize("variant,kw", [("fused", {}), ("ras", dict(tile=(8, 8, 8), k=2, overlap=1)),
                                         ("ras", dict(tile=(8, 8, 4), k=4, overlap=0))])
 def test_fp32_energy_error_3d(api, o3, variant, kw):
