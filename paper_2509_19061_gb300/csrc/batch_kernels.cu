@@ -409,8 +409,13 @@ __global__ void kb_apply_dot(const BOuter<T> *__restrict__ tab, const BSeg *__re
     const BOuter<T> &o = tab[sg.inst];
     double s0 = 0.0, s1 = 0.0;
     static_assert(BATCH_BX == AT_X && BATCH_BY == AT_Y, "batched blocks are apply tiles");
-    apply_dot_tile<T>(o.g, o.ec, o.en, o.ax, o.ay, o.px, o.py, o.qx, o.qy, o.rx, o.ry, (lb % sg.bxb) * BATCH_BX,
-                      (lb / sg.bxb) * BATCH_BY, (int)(threadIdx.y * BATCH_BX + threadIdx.x), sm, s0, s1);
+    const int i0 = (lb % sg.bxb) * BATCH_BX, j0 = (lb / sg.bxb) * BATCH_BY;
+    const int tid = (int)(threadIdx.y * BATCH_BX + threadIdx.x);
+    const size_t q = inner_entry(o.g, j0 + (int)threadIdx.y, i0 + (int)threadIdx.x);
+    const T rxq = o.rx[q], ryq = o.ry[q];
+    const TileLoad<T> l = tile_load<T>(o.g, o.ec, o.en, o.ax, o.ay, o.px, o.py, i0, j0, tid);
+    tile_flux(o.g, l, o.ax != nullptr, i0, j0, tid, sm);
+    apply_dot_cell<T>(o.g, l.vxc, l.vyc, rxq, ryq, o.qx, o.qy, i0, j0, tid, sm, s0, s1);
     block_store2(s0, s1, partials);
 }
 
