@@ -885,7 +885,7 @@ int enqueue_precond(const Precond<To, Ti> &P, int Lmax, int count, const int *li
     CK(batch_dense<Ti>(P.dense, count, P.rows, live, s));
     *nk += 3;
     for (int l = Lmax - 2; l >= 0; --l) {
-        CK(batch_prolong<Ti>(P.mid[l], P.fine[l].map, P.fine[l].nseg, P.fine[l].nblocks, live, s));
+        CK(batch_prolong<Ti>(P.mid[l], P.coarse[l].map, P.coarse[l].nseg, P.coarse[l].nblocks, live, s));
         ++*nk;
         ST(run_group<Ti>(P.grp[l][1][0], live, run, s, nk));
         ST(run_group<Ti>(P.grp[l][1][1], live, run, s, nk));

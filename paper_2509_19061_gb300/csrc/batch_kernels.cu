@@ -188,6 +188,7 @@ __global__ void kb_restrict(const BLevel<T> *__restrict__ tab, const BSeg *__res
                    p.j, p.i);
 }
 
+// (over the coarse cells)
 template <typename T>
 __global__ void kb_prolong(const BLevel<T> *__restrict__ tab, const BSeg *__restrict__ m, int n,
                             const int *__restrict__ active)
@@ -195,8 +196,8 @@ __global__ void kb_prolong(const BLevel<T> *__restrict__ tab, const BSeg *__rest
     const Pt p = point_of(m, n);
     if (!p.valid || (active && !active[p.inst])) return;
     const BLevel<T> &l = tab[p.inst];
-    prolong_point(l.g.nx, l.g.ny, l.g.pitch, l.cnx, l.cny, l.cp, (const T *)l.cvx, (const T *)l.cvy, l.vx, l.vy,
-                  p.j, p.i);
+    if (p.i < l.cnx && p.j < l.cny)
+        prolong_cell(l.g.pitch, l.cnx, l.cny, l.cp, (const T *)l.cvx, (const T *)l.cvy, l.vx, l.vy, p.j, p.i);
 }
 
 template <typename T>
@@ -363,32 +364,32 @@ template <typename T>
 __global__ void kb_residual_energy(const BOuter<T> *__restrict__ tab, const BSeg *__restrict__ m, int n,
                                    double *__restrict__ partials)
 {
+    __shared__ ApplyTile<T> sm;
     const Pt p = point_of(m, n);
     double s0 = 0.0, s1 = 0.0;
+    const BOuter<T> &o = tab[p.inst];
+    const GridDesc<T> &g = o.g;
+    const int i = p.i, j = p.j, tx = (int)threadIdx.x, ty = (int)threadIdx.y;
+    const size_t q = (size_t)j * g.pitch + i, q0 = inner_entry(g, j, i);
+    const T bx = o.bx[q0], by = o.by[q0], fx = o.fx[q0], fy = o.fy[q0], wx = -o.ivx[q0], wy = -o.ivy[q0];
+    flux_tile_stage<T>(g, o.ec, o.en, nullptr, nullptr, o.vx, o.vy, i - tx, j - ty, ty * BATCH_BX + tx, sm);
     if (p.valid) {
-        const BOuter<T> &o = tab[p.inst];
-        const GridDesc<T> &g = o.g;
-        const int i = p.i, j = p.j;
-        const size_t q = (size_t)j * g.pitch + i;
-        T mm, d, vc;
         CellSq<T> c0(s0), c1(s1); // the cell's vx and vy terms
         if (j < g.ny) {
             T r = T(0);
             if (vx_unknown(g, j, i)) {
-                op_x(g, o.ec, o.en, (const T *)o.vx, (const T *)o.vy, j, i, mm, d, vc);
-                r = r_sub(o.bx[q], mm);
-                c0.add(r, -o.ivx[q]);
-                c1.add(o.fx[q], -o.ivx[q]);
+                r = r_sub(bx, tile_mx(sm, ty, tx));
+                c0.add(r, wx);
+                c1.add(fx, wx);
             }
             o.rx[q] = r;
         }
         if (i < g.nx) {
             T r = T(0);
             if (vy_unknown(g, j, i)) {
-                op_y(g, o.ec, o.en, (const T *)o.vx, (const T *)o.vy, j, i, mm, d, vc);
-                r = r_sub(o.by[q], mm);
-                c0.add(r, -o.ivy[q]);
-                c1.add(o.fy[q], -o.ivy[q]);
+                r = r_sub(by, tile_my(sm, ty, tx));
+                c0.add(r, wy);
+                c1.add(fy, wy);
             }
             o.ry[q] = r;
         }

@@ -79,65 +79,14 @@ __global__ void k_residual(GridDesc<T> g, const T *__restrict__ ec, const T *__r
     }
 }
 
-// fine += P coarse at the fine unknowns (prolong_point's sums).  A thread takes
-// the 2 x 2 fine cells of a coarse cell: they share the coarse values (12 loads
-// for 8 points, 24 a point at a time) and the fine rows move as pairs, at even
-// columns of an even pitch.  All levels of a V-cycle on 4096^2: 79 us, 148 a
-// point at a time.
-template <typename T>
-struct alignas(2 * sizeof(T)) FinePair {
-    T e[2];
-};
+// fine += P coarse at the fine unknowns
 template <typename T>
 __global__ void __launch_bounds__(BX *BY) k_prolong_add(int fp, int ncx, int ncy, int cp, const T *__restrict__ cx,
                                                         const T *__restrict__ cy, T *__restrict__ fx,
                                                         T *__restrict__ fy)
 {
     const int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * BY + threadIdx.y;
-    if (I >= ncx || J >= ncy) return;
-    const T c34 = T(0.75), c14 = T(0.25), c12 = T(0.5);
-    const int W = I > 0 ? I - 1 : 0, E = I < ncx - 1 ? I + 1 : I; // mirrored at the walls
-    const int S = J > 0 ? J - 1 : 0, N = J < ncy - 1 ? J + 1 : J;
-    const size_t c = (size_t)J * cp, q = (size_t)(2 * J) * fp + 2 * I;
-    FinePair<T> *const px[2] = {(FinePair<T> *)(fx + q), (FinePair<T> *)(fx + q + fp)};
-    FinePair<T> *const py[2] = {(FinePair<T> *)(fy + q), (FinePair<T> *)(fy + q + fp)};
-    const FinePair<T> x0 = *px[0], x1 = *px[1], y0 = *py[0], y1 = *py[1];
-    // vx: cell-centred in y, node-centred in x
-    const T xc[2] = {cx[c + I], cx[c + I + 1]};
-    const T xo[2][2] = {{cx[(size_t)S * cp + I], cx[(size_t)S * cp + I + 1]},
-                        {cx[(size_t)N * cp + I], cx[(size_t)N * cp + I + 1]}};
-    // vy: node-centred in y, cell-centred in x
-    const T yc[2][3] = {{cy[c + W], cy[c + I], cy[c + E]}, {cy[c + cp + W], cy[c + cp + I], cy[c + cp + E]}};
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        T s = r_add(T(0), r_mul(c34, xc[0]));
-        const T even = r_add(s, r_mul(c14, xo[r][0]));
-        s = r_add(T(0), r_mul(r_mul(c34, c12), xc[0]));
-        s = r_add(s, r_mul(r_mul(c34, c12), xc[1]));
-        s = r_add(s, r_mul(r_mul(c14, c12), xo[r][0]));
-        const T odd = r_add(s, r_mul(r_mul(c14, c12), xo[r][1]));
-        const FinePair<T> x = r ? x1 : x0;
-        const FinePair<T> v = {{r_add(x.e[0], even), r_add(x.e[1], odd)}};
-        if (I > 0) *px[r] = v;
-        else px[r]->e[1] = v.e[1];
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        if (r == 0 && J == 0) continue; // the wall
-        const T w = r ? c12 : T(1);
-        FinePair<T> v = r ? y1 : y0;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            T s = r_add(T(0), r_mul(r_mul(w, c34), yc[0][1]));
-            s = r_add(s, r_mul(r_mul(w, c14), yc[0][2 * k]));
-            if (r) {
-                s = r_add(s, r_mul(r_mul(w, c34), yc[1][1]));
-                s = r_add(s, r_mul(r_mul(w, c14), yc[1][2 * k]));
-            }
-            v.e[k] = r_add(v.e[k], s);
-        }
-        *py[r] = v;
-    }
+    if (I < ncx && J < ncy) prolong_cell(fp, ncx, ncy, cp, cx, cy, fx, fy, J, I);
 }
 
 // coarse b = P^T r / 4 at the coarse unknowns (gather form), zero elsewhere
