@@ -70,13 +70,16 @@ __device__ __forceinline__ double warp_sum(double v)
 __device__ __forceinline__ void block_store2(double s0, double s1, double *partials)
 {
     __shared__ double sh[2][NT / 32];
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
+    // Both sums in one tree: after lanes l and l + 16 have been added (lanes below
+    // 16 hold s0, the others s1), the rest is per half: five FP64 additions a warp
+    // instead of ten, where the reduction is a third of a tile's FP64 work; each
+    // sum's pairs are those of warp_sum.
     const int t = threadIdx.y * BATCH_BX + threadIdx.x, lane = t & 31, wid = t >> 5;
-    if (lane == 0) {
-        sh[0][wid] = s0;
-        sh[1][wid] = s1;
-    }
+    const bool hi = lane >= 16;
+    double v = (hi ? s1 : s0) + __shfl_xor_sync(0xffffffffu, hi ? s0 : s1, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, 16);
+    if ((lane & 15) == 0) sh[lane >> 4][wid] = v;
     __syncthreads();
     if (t < 2) {
         double s = 0.0;
