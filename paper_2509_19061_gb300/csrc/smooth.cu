@@ -35,6 +35,42 @@ int stream_passes_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &ru
     else return stream64_passes(g, p.sweeps, run);
 }
 
+// The tiles of an FP32 RAS schedule that equals global Jacobi, on grids between
+// the cluster's and the row streaming's: the given tiles, shifts and k change no
+// value there, so they are chosen for this GPU.  Windows are 64 columns wide (two
+// per lane of the pair kernel) and of 5 rows a warp, a pass runs up to eight
+// sweeps, split evenly, on tiles cut at zero.  Such a grid has few tiles and a
+// launch takes the time of one times the waves: about 32 rows' worth of setup and
+// the window's rows (8.9 us with 50 rows and eight sweeps, 11.4 with 80; 32 x 32
+// tiles with k = 4 6.5 for four), so the window height with the least product is
+// taken.  With the middle levels' tiles as given: 512^2 Uzawa (32 x 32, k = 4)
+// 25.0 ms, now 24.1; 8 CG cycles of 1024^2 (48 x 32, k = 8) 7.28 and 7.11.
+constexpr long long FREE_MAX_CELLS = 600000; // where the row streaming starts
+template <typename T>
+SmoothSpec tiles_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
+{
+    if (sizeof(T) != 4 || p.variant != STOKES_RAS || p.sweeps < 1 || !any_traversal(p) || !run.allow_tma ||
+        run.pair_mode != 1 || p.k > 8 || g.nx < 64 || g.ny < 40 || (long long)g.nx * g.ny >= FREE_MAX_CELLS)
+        return p;
+    SmoothSpec q = p;
+    const int passes = (p.sweeps + 7) / 8;
+    q.k = (p.sweeps + passes - 1) / passes;
+    q.overlap = q.k - 1;
+    q.shift_mode = STOKES_SHIFT_NONE;
+    q.ti = 64 - 2 * q.k;
+    long long best = 0;
+    for (int rows : {40, 50, 65, 80}) {
+        const int tj = rows - 2 * q.k;
+        const long long tiles = (long long)((g.nx + q.ti - 1) / q.ti) * ((g.ny + tj - 1) / tj);
+        const long long cost = (tiles + 151) / 152 * (32 + rows);
+        if (best == 0 || cost < best) {
+            best = cost;
+            q.tj = tj;
+        }
+    }
+    return q;
+}
+
 } // namespace
 
 // number of ping-pong passes of a smoothing (one per sweep; one per outer
@@ -45,7 +81,8 @@ int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
     if (p.sweeps <= 0) return 0;
     if (takes_cluster(g, p, run)) return 1;
     if (const int n = stream_passes_of(g, p, run)) return n;
-    if (p.variant == STOKES_RAS) return (p.sweeps + p.k - 1) / p.k;
+    const int k = tiles_of(g, p, run).k;
+    if (p.variant == STOKES_RAS) return (p.sweeps + k - 1) / k;
     return p.sweeps;
 }
 
@@ -63,14 +100,16 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
         if (st != STOKES_OK) return st;                                                                            \
     } while (0)
     if (p.sweeps == 0) return STOKES_OK;
-    const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + p.k - 1) / p.k : 0;
+    const SmoothSpec q = tiles_of(g, p, run); // what the tile launches run
+    const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + q.k - 1) / q.k : 0;
     const bool cluster = takes_cluster(g, p, run);
     const int n_stream = stream_passes_of(g, p, run);
     const int kind = p.variant == STOKES_RAS    ? STOKES_K_RAS
                      : p.variant == STOKES_RBGS ? STOKES_K_RBGS
                                                 : STOKES_K_JACOBI;
-    if ((cluster || n_stream > 0) && p.variant == STOKES_RAS && p.shift_mode == STOKES_SHIFT_LIST)
-        for (int t = 0; t < n_outer; ++t) // the shifts change nothing, but bad ones stay refused
+    if ((cluster || n_stream > 0 || q.shift_mode != p.shift_mode) && p.variant == STOKES_RAS &&
+        p.shift_mode == STOKES_SHIFT_LIST)
+        for (int t = 0; t < (p.sweeps + p.k - 1) / p.k; ++t) // the shifts change nothing, but bad ones stay refused
             if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 || p.shifts[2 * t + 1] >= p.tj)
                 return STOKES_ERR_ARG;
     if (cluster) {
@@ -119,18 +158,18 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
         }
     } else if (p.variant == STOKES_RAS) {
         for (int t = 0; t < n_outer; ++t) {
-            const int ks = (t == n_outer - 1) ? p.sweeps - (n_outer - 1) * p.k : p.k;
+            const int ks = (t == n_outer - 1) ? q.sweeps - (n_outer - 1) * q.k : q.k;
             int si = 0, sj = 0;
-            if (p.shift_mode == STOKES_SHIFT_SPLITMIX) {
-                si = (int)(splitmix64(p.seed, 2u * (uint64_t)t) % (uint64_t)p.ti);
-                sj = (int)(splitmix64(p.seed, 2u * (uint64_t)t + 1u) % (uint64_t)p.tj);
-            } else if (p.shift_mode == STOKES_SHIFT_LIST) {
-                si = p.shifts[2 * t];
-                sj = p.shifts[2 * t + 1];
-                if (si < 0 || si >= p.ti || sj < 0 || sj >= p.tj) return STOKES_ERR_ARG;
+            if (q.shift_mode == STOKES_SHIFT_SPLITMIX) {
+                si = (int)(splitmix64(q.seed, 2u * (uint64_t)t) % (uint64_t)q.ti);
+                sj = (int)(splitmix64(q.seed, 2u * (uint64_t)t + 1u) % (uint64_t)q.tj);
+            } else if (q.shift_mode == STOKES_SHIFT_LIST) {
+                si = q.shifts[2 * t];
+                sj = q.shifts[2 * t + 1];
+                if (si < 0 || si >= q.ti || sj < 0 || sj >= q.tj) return STOKES_ERR_ARG;
             }
-            const TileGrid tg = make_tiles(g.nx, g.ny, p.ti, p.tj, si, sj);
-            LAUNCH(STOKES_K_RAS, 1, launch_ras<T>(g, k, omega, tg, ks, p.overlap, ax, ay, bx, by, run, s));
+            const TileGrid tg = make_tiles(g.nx, g.ny, q.ti, q.tj, si, sj);
+            LAUNCH(STOKES_K_RAS, 1, launch_ras<T>(g, k, omega, tg, ks, q.overlap, ax, ay, bx, by, run, s));
             ++passes;
             advance();
         }

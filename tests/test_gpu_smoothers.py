@@ -784,6 +784,32 @@ def test_rbgs_streaming_equals_the_tile_kernel(api, nx, ny, sweeps, square):
     assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
 
 
+@pytest.mark.parametrize("nx,ny,square", [(64, 257, True), (130, 127, False), (340, 96, True), (511, 333, False),
+                                          (777, 771, True)])
+def test_exact_schedules_choose_their_tiles(api, nx, ny, square):
+    """RAS with overlap >= k - 1 in FP32 on grids between the cluster and the row
+    streaming: one and several passes, even and odd, windows of every height and
+    one or more waves, with a pressure and moving walls, value for value the
+    given tiles'; a shift outside the given tile is still refused."""
+    prob = rand_problem(nx, ny, 95, lx=1.0, ly=ny / nx if square else 0.7)
+    vx, vy = inputs.random_velocity(nx, ny, 96, 0.1)
+    vx[:, 0], vx[:, nx], vy[0], vy[ny] = 0.3, -0.2, 0.1, 0.4
+    p = inputs.random_pressure(nx, ny, 97)
+    for sweeps in (1, 5, 8, 13, 23):
+        outs = []
+        for pair in (0, 1):
+            r = Run(api, prob, "f32", (vx, vy), p)
+            r.ctx.set_option(api.STOKES_OPT_PAIRED, pair)
+            r.smooth(variant="ras", sweeps=sweeps, tile=(32, 24), k=4, overlap=3, seed=7)
+            outs.append(r.v())
+            if pair:
+                with pytest.raises(api.StokesError) as e:
+                    r.smooth(variant="ras", sweeps=5, tile=(32, 24), k=4, overlap=3, shifts=[[0, 0], [0, 24]])
+                assert e.value.status == api.STOKES_ERR_ARG
+            r.ctx.close()
+        assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("kw", [
     dict(variant="jacobi", sweeps=3), dict(variant="fused", sweeps=3), dict(variant="rbgs", sweeps=2),
