@@ -257,9 +257,11 @@ __global__ void __launch_bounds__(RB_MAX * 32, RB_CTAS) k_rbgs_stream(const __gr
 
 int rbgs_stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run)
 {
-    if (!run.allow_tma || run.pair_mode != 1 || sweeps < 1) return 0;
-    // (20 sweeps: 512^2 171 us either way, 768^2 207 and 253 by tiles)
-    if ((long long)g.nx * g.ny < RB_MIN_CELLS) return 0;
+    // One sweep, or two on the smaller grids, gain less than the copy back that an
+    // odd pass count costs: 8192^2 one sweep 1014 us, 962 by tiles; two at 640^2
+    // 28.4 and 26.4, at 1024^2 37.9 and 39.7.
+    const long long least = sweeps == 2 ? 2 * RB_MIN_CELLS : RB_MIN_CELLS;
+    if (!run.allow_tma || run.pair_mode != 1 || sweeps < 2 || (long long)g.nx * g.ny < least) return 0;
     return (sweeps + RB_MAX - 1) / RB_MAX;
 }
 
