@@ -324,9 +324,9 @@ TILE_KERNEL_NAMES = {"pair": "k_ras_pair", "tma": "k_ras_tma", "global": "k_ras_
 
 def tile_kernel_name(api, n, tile, k, overlap, dt_name):
     """Name of the kernel the library picks for this schedule: row streaming
-    where it equals global Jacobi on a large FP32 grid, else a tile kernel."""
-    if dt_name == "f32" and overlap >= k - 1 and n * n >= 600000:
-        return "k_ras_stream"
+    where it equals global Jacobi on a large grid, else a tile kernel."""
+    if overlap >= k - 1 and n * n >= (600000 if dt_name == "f32" else 100000):
+        return "k_ras_stream" if dt_name == "f32" else "k_ras_stream64"
     return TILE_KERNEL_NAMES[api.stokes_tile_kernel_plan(n, n, tuple(tile), overlap, dt_name)[0]]
 
 
@@ -543,12 +543,15 @@ def e2e_measure(args, ctx, prob, stream, world, barrier=lambda: None):
     steps = max(2, args.steps)
 
     def h2d(i):
-        # buffer set i % 2 is free once step i - 2's result has left it
+        # buffer set i % 2: the viscosity and the force are free once step i - 2
+        # has computed, the velocity once its result has left
         b = dev[i % 2]
         with torch.cuda.stream(cs):
             if i >= 2:
-                cs.wait_event(drained[i % 2])
+                cs.wait_event(computed[i % 2])
             for name, t in host.items():
+                if name == "vx" and i >= 2:
+                    cs.wait_event(drained[i % 2])
                 b[name].copy_(t, non_blocking=True)
             copied[i % 2].record(cs)
 
