@@ -199,12 +199,14 @@ int stokes_apply_operator(stokes_ctx *ctx, const void *vx, const void *vy, const
  * (Sec. 5).  p may be NULL (p = 0).  Requires stokes_set_viscosity and
  * stokes_set_rhs.  Asynchronous.  The passes ping-pong between (vx, vy) and
  * context-owned scratch fields; the first call whose pass count is odd and at
- * least 3 (RAS: ceil(sweeps / k) outer iterations, Jacobi variants:
- * one pass per sweep; large FP32 schedules with o >= k - 1, and fused Jacobi,
- * run passes of up to eight sweeps instead) allocates a second scratch pair (two fields) so that the result
+ * least 3 allocates a second scratch pair (two fields) so that the result
  * ends in (vx, vy) without a copy: make that call once before capturing
  * stokes_smooth into a CUDA graph.  Returns STOKES_ERR_OOM if that allocation
- * fails. */
+ * fails.  Passes: RAS ceil(sweeps / k) outer iterations, the Jacobi variants and
+ * RBGS one per sweep.  Where the result is the same value for value, fewer run:
+ * RAS with o >= k - 1 (any shifts) and fused Jacobi up to eight sweeps a pass on
+ * large grids and all sweeps in one launch, in place, on small ones; RBGS in FP32
+ * two sweeps a pass on large grids. */
 int stokes_smooth(stokes_ctx *ctx, void *vx, void *vy, const void *p, const stokes_smooth_params *params);
 
 /* Energy residual sums of Sec. 6.4, accumulated in FP64:
@@ -305,7 +307,10 @@ typedef enum {
                                         instructions); 2: every FP32 window of at most 64 columns
                                         does; 0: never (one column per thread).  Needs
                                         STOKES_OPT_USE_TMA; the results are identical either way
-                                        (up to the sign of exact zeros).  Other values:
+                                        (up to the sign of exact zeros).  With 1 (and
+                                        STOKES_OPT_USE_TMA) schedules that equal global Jacobi,
+                                        and RBGS, also take the row-streaming and one-launch
+                                        kernels; 0 and 2 keep them on tiles.  Other values:
                                         STOKES_ERR_ARG. */
 } stokes_option;
 

@@ -165,7 +165,8 @@ __global__ void k_assemble(const DenseJob *__restrict__ jobs)
 // divisions, not by bytes (n^2 doubles stay in L2).  One CTA per matrix kept
 // one SM's FP64 pipe for the whole n^3 / 6: 12.4 ms for L and 12.5 ms for W at
 // n = 480.  Blocked by 32 columns the work spreads over the SMs and only the
-// chain stays serial: 0.86 and 0.43 ms (and 0.065 for W^T W, from 0.157).  Every entry is still formed by the same operations in
+// chain stays serial: 0.71 and 0.43 ms (and 0.065 for W^T W, from 0.157).  Every
+// entry is still formed by the same operations in
 // the same order (its updates in ascending k, then its division), so the
 // factors have the bits of the unblocked algorithm.
 constexpr int DN_B = 32;  // block columns
