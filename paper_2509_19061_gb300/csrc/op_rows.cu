@@ -197,6 +197,11 @@ __device__ __forceinline__ void op_band(const OpRows<T> &o, int strip, int j0, i
             sy = r_mul(sh, g.ihx);
         }
     };
+    // FP32 levels of a few rows wait for memory only, so row j0 is in flight with
+    // the rows before it (the smallest
+    // levels: 6.3 us, 5.1 so and with bands of one coarse row); FP64 keeps the registers.
+    OpRow<T> cur;
+    if (sizeof(T) == 4) cur = load(j0);
     // state at row j: velocity, scaled shear at its nodes, Tyy and p of the row before
     V2<T> vx, vy, sx, sy, ty, ps = {{T(0), T(0)}};
     {
@@ -215,7 +220,7 @@ __device__ __forceinline__ void op_band(const OpRows<T> &o, int strip, int j0, i
         if (hasp) ps = r.p;
     }
     Restrict<T> acc = {T(0), T(0), T(0)};
-    OpRow<T> cur = load(j0);
+    if (sizeof(T) == 8) cur = load(j0);
     for (int j = j0; j < j1; ++j) {
         OpRow<T> nxt = cur;
         if (j + 1 < j1) nxt = load(j + 1);
@@ -286,12 +291,12 @@ __global__ void __launch_bounds__(OR_THREADS, OR_BLOCKS<T>) k_op_rows(const __gr
 }
 
 // bands of one warp each, as many as one wave holds but at least four rows
-// (two coarse rows); columns 0 .. cols - 1
+// (one coarse row); columns 0 .. cols - 1
 template <int MODE, typename T>
 cudaError_t run(OpRows<T> &o, int cols, cudaStream_t s)
 {
     o.strips = (cols + OR_OWN - 1) / OR_OWN;
-    const int nrow = MODE == OR_RESTRICT ? o.g.ny / 2 + 1 : o.g.ny + 1, least = MODE == OR_RESTRICT ? 2 : 4;
+    const int nrow = MODE == OR_RESTRICT ? o.g.ny / 2 + 1 : o.g.ny + 1, least = MODE == OR_RESTRICT ? 1 : 4;
     const int bands = std::max(1, std::min(152 * OR_BLOCKS<T> * OR_WARPS / o.strips, (nrow + least - 1) / least));
     o.rows = (nrow + bands - 1) / bands;
     const long long items = (long long)o.strips * ((nrow + o.rows - 1) / o.rows);
