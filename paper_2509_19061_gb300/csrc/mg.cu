@@ -28,7 +28,7 @@ struct MgHierarchy {
     void *vel = nullptr;  // vx, vy of every level, back to back: one memset zeroes them all
     size_t vel_bytes = 0;
     int n = 0; // coarsest unknowns
-    double *A = nullptr, *W = nullptr, *Ainv = nullptr, *bvec = nullptr, *xvec = nullptr;
+    double *A = nullptr, *W = nullptr, *Ainv = nullptr;
     int *dstatus = nullptr;
     const void *zx = nullptr, *zy = nullptr; // finest-level result of the last enqueued application
 };
@@ -46,10 +46,10 @@ void free_level(MgLevel &l)
 void free_all(MgHierarchy *h)
 {
     for (int l = 0; l < h->L; ++l) free_level(h->lv[l]);
-    void *ps[] = {h->A, h->W, h->Ainv, h->bvec, h->xvec, h->dstatus, h->vel};
+    void *ps[] = {h->A, h->W, h->Ainv, h->dstatus, h->vel};
     for (void *p : ps)
         if (p) cudaFree(p);
-    h->A = h->W = h->Ainv = h->bvec = h->xvec = nullptr;
+    h->A = h->W = h->Ainv = nullptr;
     h->dstatus = nullptr;
     h->vel = nullptr;
     h->L = 0;
@@ -165,8 +165,7 @@ int build(MgHierarchy *h, const MgOuter &o, int levels, int coarsest, cudaStream
     h->n = n_unknowns(lc.nx, lc.ny);
     const size_t nn = (size_t)h->n * h->n;
     if (cudaMalloc(&h->A, nn * 8) != cudaSuccess || cudaMalloc(&h->W, nn * 8) != cudaSuccess ||
-        cudaMalloc(&h->Ainv, nn * 8) != cudaSuccess || cudaMalloc(&h->bvec, h->n * 8) != cudaSuccess ||
-        cudaMalloc(&h->xvec, h->n * 8) != cudaSuccess || cudaMalloc(&h->dstatus, sizeof(int)) != cudaSuccess)
+        cudaMalloc(&h->Ainv, nn * 8) != cudaSuccess || cudaMalloc(&h->dstatus, sizeof(int)) != cudaSuccess)
         return STOKES_ERR_OOM;
     CKS(cudaMemsetAsync(h->dstatus, 0, sizeof(int), s));
     CKS(mg_dense_setup<Ti>(lc, h->n, h->A, h->W, h->Ainv, h->dstatus, s));
@@ -281,7 +280,7 @@ int enqueue_precond(MgHierarchy *h, const Tc *rx, const Tc *ry, Tc *zx, Tc *zy, 
                mg_residual_restrict<Ti>(f, h->lv[l + 1], s));
     }
     // coarsest: exact solve
-    LAUNCH(STOKES_K_MG, 3, mg_dense_solve<Ti>(h->lv[L - 1], h->n, h->Ainv, h->bvec, h->xvec, s));
+    LAUNCH(STOKES_K_MG, 1, mg_dense_solve<Ti>(h->lv[L - 1], h->n, h->Ainv, s));
     // up: prolong and correct, smooth
     for (int l = L - 2; l >= 0; --l) {
         MgLevel &f = h->lv[l];

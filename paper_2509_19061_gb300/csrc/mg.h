@@ -139,6 +139,6 @@ struct DenseJob {
 template <typename T>
 cudaError_t mg_dense_setup_many(const DenseJob *jobs, int count, int nmax, cudaStream_t s);
 template <typename T>
-cudaError_t mg_dense_solve(const MgLevel &l, int n, const double *Ainv, double *bvec, double *xvec, cudaStream_t s);
+cudaError_t mg_dense_solve(const MgLevel &l, int n, const double *Ainv, cudaStream_t s);
 
 } // namespace stokes
