@@ -657,6 +657,7 @@ struct Precond {
     const BLevel<Ti> *mid[B_MAX_LEVELS] = {};
     const BLevel<Ti> *fin0 = nullptr; // level 0 after its post-smoothing (z)
     Sub fine[B_MAX_LEVELS], coarse[B_MAX_LEVELS];
+    Sub rows32[B_MAX_LEVELS]; // FP32: the blocks of batch_residual_restrict
     Group<Ti> grp[B_MAX_LEVELS][2][2]; // [level][phase][single-tile, tiled]
     const BDense<Ti> *dense = nullptr;
     int rows = 0;
@@ -713,7 +714,7 @@ int plan_precond(stokes_batch *b, const stokes_mg_params *p, Precond<To, Ti> *P)
         std::vector<BLevel<Ti>> &t = tabs[l];
         t.resize(n);
         std::memset((void *)t.data(), 0, t.size() * sizeof(BLevel<Ti>));
-        std::vector<Rect> rf, rc;
+        std::vector<Rect> rf, rc, rr;
         for (int i = 0; i < n; ++i) {
             if (l >= h->L[i]) continue;
             const MgLevel v = level_view(h, l, i, es);
@@ -742,11 +743,13 @@ int plan_precond(stokes_batch *b, const stokes_mg_params *p, Precond<To, Ti> *P)
                 e.cvy = (Ti *)c.vy;
                 rf.push_back({i, v.nx + 1, v.ny + 1});
                 rc.push_back({i, c.nx + 1, c.ny + 1});
+                rr.push_back({i, (v.nx + OR_BATCH_COLS) / OR_BATCH_COLS * BATCH_BX, c.ny + 1});
             }
         }
         ST(upload(o, t, &P->lev[l], s));
         ST(make_sub(o, rf, &P->fine[l], s));
         ST(make_sub(o, rc, &P->coarse[l], s));
+        if (sizeof(Ti) == 4) ST(make_sub(o, rr, &P->rows32[l], s, OR_BATCH_WARPS * OR_BATCH_ROWS));
         std::vector<VBuf> cur(n);
         for (int i = 0; i < n; ++i) cur[i] = {t[i].vx, t[i].vy, t[i].sx, t[i].sy};
         // smoothing groups of this level: whole-level single tiles (Jacobi-like
@@ -878,9 +881,15 @@ int enqueue_precond(const Precond<To, Ti> &P, int Lmax, int count, const int *li
     for (int l = 0; l < Lmax - 1; ++l) {
         ST(run_group<Ti>(P.grp[l][0][0], live, run, s, nk));
         ST(run_group<Ti>(P.grp[l][0][1], live, run, s, nk));
-        CK(batch_residual<Ti>(P.mid[l], P.fine[l].map, P.fine[l].nseg, P.fine[l].nblocks, live, s));
-        CK(batch_restrict<Ti>(P.mid[l], P.coarse[l].map, P.coarse[l].nseg, P.coarse[l].nblocks, live, s));
-        *nk += 2;
+        if constexpr (sizeof(Ti) == 4) {
+            const Sub &r = P.rows32[l];
+            CK(batch_residual_restrict(P.mid[l], r.map, r.nseg, r.nblocks, live, s));
+            ++*nk;
+        } else {
+            CK(batch_residual<Ti>(P.mid[l], P.fine[l].map, P.fine[l].nseg, P.fine[l].nblocks, live, s));
+            CK(batch_restrict<Ti>(P.mid[l], P.coarse[l].map, P.coarse[l].nseg, P.coarse[l].nblocks, live, s));
+            *nk += 2;
+        }
     }
     CK(batch_dense<Ti>(P.dense, count, P.rows, live, s));
     *nk += 3;

@@ -19,6 +19,18 @@ struct BSeg {
     int block_begin; // first block of this instance
 };
 
+// the segment of `n` that block `b` belongs to
+__device__ __forceinline__ int seg_of(const BSeg *__restrict__ m, int n, int b)
+{
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (m[mid].block_begin <= b) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
 // one instance at one multigrid level (inner precision T)
 template <typename T>
 struct BLevel {
@@ -76,6 +88,13 @@ cudaError_t batch_residual(const BLevel<T> *tab, const BSeg *map, int nseg, int 
 template <typename T>
 cudaError_t batch_restrict(const BLevel<T> *tab, const BSeg *map, int nseg, int nblocks, const int *active,
                            cudaStream_t s);
+// Residual and restriction in one launch by row-marching warps (op_rows.cu):
+// blocks of OR_BATCH_WARPS warps, one strip of 60 columns each and
+// OR_BATCH_ROWS coarse rows a warp, so a segment's rectangle is
+// 32 x strips wide and a block OR_BATCH_WARPS x OR_BATCH_ROWS high.
+constexpr int OR_BATCH_COLS = 60, OR_BATCH_WARPS = 4, OR_BATCH_ROWS = 4;
+cudaError_t batch_residual_restrict(const BLevel<float> *tab, const BSeg *map, int nseg, int nblocks,
+                                    const int *active, cudaStream_t s);
 template <typename T>
 cudaError_t batch_prolong(const BLevel<T> *tab, const BSeg *map, int nseg, int nblocks, const int *active,
                           cudaStream_t s);

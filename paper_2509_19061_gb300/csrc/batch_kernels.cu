@@ -15,17 +15,6 @@ namespace {
 
 constexpr int NT = BATCH_BX * BATCH_BY;
 
-__device__ __forceinline__ int seg_of(const BSeg *__restrict__ m, int n, int b)
-{
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (m[mid].block_begin <= b) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 // point of this thread inside its instance's rectangle (valid = inside)
 struct Pt {
     int inst, i, j;
@@ -743,8 +732,6 @@ cudaError_t batch_scalars(int count, const double *pq_pr, const double *zq, cons
 
 #define INST(T)                                                                                                    \
     template cudaError_t batch_rhs<T>(const BRhs<T> *, const BSeg *, int, int, cudaStream_t);                      \
-    template cudaError_t batch_residual<T>(const BLevel<T> *, const BSeg *, int, int, const int *, cudaStream_t);  \
-    template cudaError_t batch_restrict<T>(const BLevel<T> *, const BSeg *, int, int, const int *, cudaStream_t);  \
     template cudaError_t batch_prolong<T>(const BLevel<T> *, const BSeg *, int, int, const int *, cudaStream_t);   \
     template cudaError_t batch_zero_v<T>(const BLevel<T> *, const BSeg *, int, int, const int *, cudaStream_t);    \
     template cudaError_t batch_copy<T>(const BLevel<T> *, const BSeg *, int, int, bool, const int *,               \
@@ -781,5 +768,9 @@ template cudaError_t batch_cast_out<float, float>(const BOuter<float> *, const B
                                                    const int *, cudaStream_t);
 template cudaError_t batch_cast_out<float, double>(const BOuter<float> *, const BLevel<double> *, const BSeg *, int, int,
                                                    const int *, cudaStream_t);
+
+// (FP32 levels form both by rows, op_rows.cu)
+template cudaError_t batch_residual<double>(const BLevel<double> *, const BSeg *, int, int, const int *, cudaStream_t);
+template cudaError_t batch_restrict<double>(const BLevel<double> *, const BSeg *, int, int, const int *, cudaStream_t);
 
 } // namespace stokes

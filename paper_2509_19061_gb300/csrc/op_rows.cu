@@ -20,12 +20,13 @@
 // columns is a lane's first, and the coarse sums gather their fine rows in
 // ascending order, so they accumulate as the march passes and the residual
 // never goes to memory.  FP32 is bound by its loads.  All levels of a V-cycle on
-// 4096^2: 153 us, 328 as a residual and a restriction a level.
+// 4096^2: 149 us, 328 as a residual and a restriction a level.
 //
 // Operations and their order are those of stencil.cuh, so M v has the bits of
 // the other kernels.
 #include <algorithm>
 
+#include "batch.h"
 #include "internal.h"
 #include "stencil.cuh"
 
@@ -198,8 +199,8 @@ __device__ __forceinline__ void op_band(const OpRows<T> &o, int strip, int j0, i
         }
     };
     // FP32 levels of a few rows wait for memory only, so row j0 is in flight with
-    // the rows before it (the smallest
-    // levels: 6.3 us, 5.1 so and with bands of one coarse row); FP64 keeps the registers.
+    // the rows before it (the smallest levels: 6.3 us, 5.1 so and with bands of one
+    // coarse row); FP64 keeps the registers.
     OpRow<T> cur;
     if (sizeof(T) == 4) cur = load(j0);
     // state at row j: velocity, scaled shear at its nodes, Tyy and p of the row before
@@ -290,6 +291,37 @@ __global__ void __launch_bounds__(OR_THREADS, OR_BLOCKS<T>) k_op_rows(const __gr
     }
 }
 
+// The residual and its restriction of every instance of a batch, in FP32: 24
+// launches over 64 instances of 64^2 to 1024^2 took 1012 us for the residuals, a
+// thread per unknown, and 525 for the restrictions, and take 666 here.
+static_assert(OR_BATCH_COLS == OR_OWN && OR_BATCH_WARPS == OR_WARPS, "a block's strip and warps");
+__global__ void __launch_bounds__(OR_THREADS, OR_BLOCKS<float>)
+    k_op_rows_batch(const BLevel<float> *__restrict__ tab, const BSeg *__restrict__ m, int nseg,
+                    const int *__restrict__ active)
+{
+    const BSeg sg = m[seg_of(m, nseg, (int)blockIdx.x)];
+    if (active && !active[sg.inst]) return;
+    const BLevel<float> &l = tab[sg.inst];
+    OpRows<float> o;
+    o.g = l.g;
+    o.ec = l.ec;
+    o.en = l.en;
+    o.vx = l.vx;
+    o.vy = l.vy;
+    o.p = nullptr;
+    o.bx = l.bx;
+    o.by = l.by;
+    o.ox = l.cbx;
+    o.oy = l.cby;
+    o.cp = l.cp;
+    const int lb = (int)blockIdx.x - sg.block_begin, strip = lb % sg.bxb;
+    const int r0 = (lb / sg.bxb * OR_WARPS + (int)threadIdx.x / 32) * OR_BATCH_ROWS, nrow = o.g.ny / 2 + 1;
+    if (r0 >= nrow) return; // (the whole warp)
+    const int r1 = min(r0 + OR_BATCH_ROWS, nrow), j0 = max(2 * r0 - 1, 0), j1 = min(2 * r1, o.g.ny) + 1;
+    if (o.g.square) op_band<OR_RESTRICT, true>(o, strip, j0, j1, r0, r1);
+    else op_band<OR_RESTRICT, false>(o, strip, j0, j1, r0, r1);
+}
+
 // bands of one warp each, as many as one wave holds but at least four rows
 // (one coarse row); columns 0 .. cols - 1
 template <int MODE, typename T>
@@ -365,5 +397,12 @@ template cudaError_t op_rows_restrict<float>(const GridDesc<float> &, const floa
 template cudaError_t op_rows_restrict<double>(const GridDesc<double> &, const double *, const double *,
                                               const double *, const double *, const double *, const double *,
                                               double *, double *, int, cudaStream_t);
+
+cudaError_t batch_residual_restrict(const BLevel<float> *tab, const BSeg *map, int nseg, int nblocks,
+                                    const int *active, cudaStream_t s)
+{
+    if (nblocks > 0) k_op_rows_batch<<<nblocks, OR_THREADS, 0, s>>>(tab, map, nseg, active);
+    return cudaGetLastError();
+}
 
 } // namespace stokes

@@ -234,7 +234,8 @@ def test_batched_defect_correction_is_bitwise_the_single_context(api, dtype, inn
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 def test_single_transfers_are_bitwise_the_batched_points(api, dtype):
     """A single V-cycle forms the residual with its restriction by rows (levels
-    of FP64 from 100000 cells, of FP32 all); the batch takes a point at a time.  Levels whose columns end on, before and
+    of FP64 from 100000 cells, of FP32 all); the batch does so in FP32 with other
+    bands, and takes a point at a time in FP64.  Levels whose columns end on, before and
     after a strip of 60 (30 coarse), few and many rows, both cell shapes."""
     import torch
     probs = [inputs.sinker_problem(nx, ny, eta_in=1e2, lx=1.0, ly=r * ny / nx)
