@@ -657,6 +657,7 @@ struct Precond {
     const BLevel<Ti> *mid[B_MAX_LEVELS] = {};
     const BLevel<Ti> *fin0 = nullptr; // level 0 after its post-smoothing (z)
     Sub fine[B_MAX_LEVELS], coarse[B_MAX_LEVELS];
+    Sub zero[B_MAX_LEVELS];   // the blocks of batch_zero_v
     Sub rows32[B_MAX_LEVELS]; // FP32: the blocks of batch_residual_restrict
     Group<Ti> grp[B_MAX_LEVELS][2][2]; // [level][phase][single-tile, tiled]
     const BDense<Ti> *dense = nullptr;
@@ -714,7 +715,7 @@ int plan_precond(stokes_batch *b, const stokes_mg_params *p, Precond<To, Ti> *P)
         std::vector<BLevel<Ti>> &t = tabs[l];
         t.resize(n);
         std::memset((void *)t.data(), 0, t.size() * sizeof(BLevel<Ti>));
-        std::vector<Rect> rf, rc, rr;
+        std::vector<Rect> rf, rc, rr, rz;
         for (int i = 0; i < n; ++i) {
             if (l >= h->L[i]) continue;
             const MgLevel v = level_view(h, l, i, es);
@@ -743,12 +744,15 @@ int plan_precond(stokes_batch *b, const stokes_mg_params *p, Precond<To, Ti> *P)
                 e.cvy = (Ti *)c.vy;
                 rf.push_back({i, v.nx + 1, v.ny + 1});
                 rc.push_back({i, c.nx + 1, c.ny + 1});
+                const size_t words = (size_t)(v.ny + 1) * v.pitch * sizeof(Ti) / 16;
+                rz.push_back({i, 1, (int)((words + ZERO_BLOCK - 1) / ZERO_BLOCK)});
                 rr.push_back({i, (v.nx + OR_BATCH_COLS) / OR_BATCH_COLS * BATCH_BX, c.ny + 1});
             }
         }
         ST(upload(o, t, &P->lev[l], s));
-        ST(make_sub(o, rf, &P->fine[l], s));
+        if (sizeof(Ti) == 8) ST(make_sub(o, rf, &P->fine[l], s));
         ST(make_sub(o, rc, &P->coarse[l], s));
+        ST(make_sub(o, rz, &P->zero[l], s, 1));
         if (sizeof(Ti) == 4) ST(make_sub(o, rr, &P->rows32[l], s, OR_BATCH_WARPS * OR_BATCH_ROWS));
         std::vector<VBuf> cur(n);
         for (int i = 0; i < n; ++i) cur[i] = {t[i].vx, t[i].vy, t[i].sx, t[i].sy};
@@ -875,7 +879,7 @@ int enqueue_precond(const Precond<To, Ti> &P, int Lmax, int count, const int *li
         ++*nk;
     }
     for (int l = 0; l < Lmax - 1; ++l) {
-        CK(batch_zero_v<Ti>(P.lev[l], P.fine[l].map, P.fine[l].nseg, P.fine[l].nblocks, live, s));
+        CK(batch_zero_v<Ti>(P.lev[l], P.zero[l].map, P.zero[l].nseg, P.zero[l].nblocks, live, s));
         ++*nk;
     }
     for (int l = 0; l < Lmax - 1; ++l) {

@@ -98,7 +98,9 @@ cudaError_t batch_residual_restrict(const BLevel<float> *tab, const BSeg *map, i
 template <typename T>
 cudaError_t batch_prolong(const BLevel<T> *tab, const BSeg *map, int nseg, int nblocks, const int *active,
                           cudaStream_t s);
-// zero v of every listed level (map over pitch x (ny+1))
+// zero v of every listed level (segments of ceil(16-byte words of a field /
+// ZERO_BLOCK) blocks)
+constexpr int ZERO_BLOCK = 1024;
 template <typename T>
 cudaError_t batch_zero_v(const BLevel<T> *tab, const BSeg *map, int nseg, int nblocks, const int *active,
                          cudaStream_t s);
