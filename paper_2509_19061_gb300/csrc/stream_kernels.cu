@@ -36,7 +36,9 @@
 // back warp reads the coefficients of its rows there again.  Their only
 // synchronisation is one barrier of the two warps per row.  A cell outside
 // the unknowns has weight zero (its 1/diag is zero), so walls and the outside
-// keep their values.
+// keep their values within a pass while the fields are finite.  Only unknowns
+// are stored: where a field overflows, the product of zero and infinity next
+// to a wall never reaches the wall's own entry in memory.
 #include <algorithm>
 
 #include "f32x2.cuh"
@@ -201,11 +203,12 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
         vx[t] = vy[t] = sx[t] = ty[t] = zero;
         if (!SQ) ay[SQ ? 0 : t] = sy[SQ ? 0 : t] = zero;
     }
-    // columns this lane writes: all four, or `part` at the grid's right end
+    // the unknowns this lane writes: all four columns, or single ones beside the
+    // west wall (vx of column 0) and at the grid's right end
     const bool mine = 4 * lane >= a.hl && 4 * lane < a.hl + a.own;
-    const bool full = mine && c0 + 4 <= nx;
-    const int part = mine && !full ? nx - c0 : 0;
-    const bool ragged = __any_sync(0xffffffffu, part > 0);
+    const bool full_y = mine && c0 + 4 <= nx, full_x = full_y && c0 > 0;
+    const int part_x = mine && !full_x ? min(nx - c0, 4) : 0, part_y = mine && !full_y ? nx - c0 : 0;
+    const bool edge = __any_sync(0xffffffffu, part_x > 0);
     int row = jb - n + (back ? KL : 0);       // row the pass completes in this step, as a back warp
     long long q = (long long)row * P + c0;
     int slot = 0;                             // staged slot of the round's first row
@@ -270,17 +273,18 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
                 *reinterpret_cast<f4 *>(out) = ix;
                 *reinterpret_cast<f4 *>(out + ST_COLS) = iy;
             } else if (row >= y0 && row < y1) {
-                st4_if(a.ox + q, ix, full);
-                st4_if(a.oy + q, iy, full);
-                if (ragged) {
-                    const f4 o[2] = {ix, iy};
-#pragma unroll
-                    for (int w = 0; w < 2; ++w) {
-                        float *const p = (w ? a.oy : a.ox) + q;
-                        if (part > 0) p[0] = f2lo(o[w].a);
-                        if (part > 1) p[1] = f2hi(o[w].a);
-                        if (part > 2) p[2] = f2lo(o[w].b);
-                    }
+                const bool uy = row > 0; // (row 0 of vy is a wall)
+                st4_if(a.ox + q, ix, full_x);
+                st4_if(a.oy + q, iy, full_y && uy);
+                if (edge) {
+                    float *const px = a.ox + q, *const py = a.oy + q;
+                    if (part_x > 0 && c0 > 0) px[0] = f2lo(ix.a);
+                    if (part_x > 1) px[1] = f2hi(ix.a);
+                    if (part_x > 2) px[2] = f2lo(ix.b);
+                    if (part_x > 3) px[3] = f2hi(ix.b);
+                    if (part_y > 0 && uy) py[0] = f2lo(iy.a);
+                    if (part_y > 1 && uy) py[1] = f2hi(iy.a);
+                    if (part_y > 2 && uy) py[2] = f2lo(iy.b);
                 }
             }
             ++row;

@@ -840,3 +840,29 @@ def test_smoothers_ignore_layout_padding(api, dtype, kw):
         r, c = b.ctx.shape[name]
         h = t.double().cpu().numpy()
         assert np.isnan(h[r:, :]).all() and np.isnan(h[:, c:]).all(), name
+
+
+@pytest.mark.parametrize("nx,ny,square", [(1121, 641, True), (901, 700, False), (3, 250001, False)])
+def test_row_streaming_keeps_the_walls_of_an_overflowing_field(api, nx, ny, square):
+    """Velocities near the largest FP32 number beside the west and south walls
+    overflow within a few sweeps: the caller's Dirichlet values stay, bit for
+    bit, and the overflow reaches the entries that it reaches in separate-pass
+    Jacobi, over one pass of sweeps and over several."""
+    prob = rand_problem(nx, ny, 61, lx=1.0, ly=ny / nx if square else 0.7)
+    vx, vy = inputs.random_velocity(nx, ny, 62, 0.1)
+    vx[ny // 3, 1], vy[1, nx // 2], vy[ny // 2, 0] = 1e38, -1e38, 1e38
+    vx[:, 0], vx[:, nx], vy[0], vy[ny] = 0.3, -0.2, 0.1, 0.4
+    for sweeps in (5, 19):
+        outs = []
+        for variant in ("jacobi", "fused"):
+            r = Run(api, prob, "f32", (vx, vy))
+            r.smooth(variant=variant, sweeps=sweeps)
+            outs.append(r.v())
+            r.ctx.close()
+        for x, y in outs:
+            assert (x[:, 0] == np.float32(0.3)).all() and (x[:, nx] == np.float32(-0.2)).all()
+            assert (y[0] == np.float32(0.1)).all() and (y[ny] == np.float32(0.4)).all()
+        for a, b in zip(*outs):
+            fin = np.isfinite(a)
+            assert not fin.all() and np.array_equal(fin, np.isfinite(b))
+            assert np.array_equal(a[fin], b[fin])
