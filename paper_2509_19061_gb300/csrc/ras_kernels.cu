@@ -636,11 +636,11 @@ __device__ __forceinline__ void pair_sweeps(const RasArgs<float> &a, const Windo
         sweep(std::integral_constant<int, 1>());
     }
     if (s < a.ks) sweep(std::integral_constant<int, 0>());
-    // ---- write back the tile's own cells.  Both components of every owned
-    // cell are stored: the cells a sweep does not update (walls) keep their
-    // staged value, which is the value already there (the walls of both
-    // buffers of a ping-pong pair are the same), and an owned cell lies
-    // inside both arrays' extents.
+    // ---- write back the unknowns of the tile's own cells, which lie inside
+    // both arrays' extents.  The walls (vx of column 0, vy of row 0) stay as
+    // they are in memory: their weight is zero, but zero times the infinity of
+    // a field that overflows is not, and the walls of a V-cycle level's buffers
+    // are zeroed once for all solves.
     const long long P = (long long)g.pitch;
     const int gx0 = w.ox0 + 2 * lane, gy0 = w.oy0 + strip * PR;
     const bool own0 = gx0 >= w.x0 && gx0 < w.x1, own1 = gx0 + 1 >= w.x0 && gx0 + 1 < w.x1;
@@ -648,14 +648,11 @@ __device__ __forceinline__ void pair_sweeps(const RasArgs<float> &a, const Windo
 #pragma unroll
     for (int r = 0; r < PR; ++r, q += P) {
         if (gy0 + r < w.y0 || gy0 + r >= w.y1) continue;
-        if (own0) {
-            a.ox[q] = f2lo(c.vx[r]);
-            a.oy[q] = f2lo(c.vy[r]);
-        }
-        if (own1) {
-            a.ox[q + 1] = f2hi(c.vx[r]);
-            a.oy[q + 1] = f2hi(c.vy[r]);
-        }
+        const bool uy = gy0 + r > 0;
+        if (own0 && gx0 > 0) a.ox[q] = f2lo(c.vx[r]);
+        if (own0 && uy) a.oy[q] = f2lo(c.vy[r]);
+        if (own1 && gx0 >= 0) a.ox[q + 1] = f2hi(c.vx[r]);
+        if (own1 && uy) a.oy[q + 1] = f2hi(c.vy[r]);
     }
 }
 

@@ -358,3 +358,28 @@ def test_full_batched_workload_samples_match_single_contexts(api, tile, k, o):
         assert np.array_equal(b.unpack(vx, "vx", i), r[0]), i
         assert np.array_equal(b.unpack(vy, "vy", i), r[1]), i
     b.close()
+
+
+def test_a_diverged_batch_solve_leaves_no_trace(api):
+    """A batched solve whose FP32 V-cycle overflows (row streaming and the pair
+    kernel) leaves nothing behind: the next one, on tiles of the one-column
+    kernel, equals that of a fresh batch bit for bit."""
+    import torch
+    probs = problems([(768, 768), (512, 512), (256, 320), (64, 64)], 31)
+    kw = dict(variant="ras", nu_max=20, inner="f32", krylov=True, tol=1e-12, max_cycles=3)
+    outs = []
+    for overflow in (False, True):
+        b = batch_context(api, probs, "f64")
+        vx, vy = b.slab(), b.slab()
+        if overflow:
+            status = b.solve(vx, vy, None, tile=(48, 64), k=8, overlap=7, omega=1e30, **kw)[3]
+            assert all(s == api.STOKES_ERR_DIVERGED for s in status)
+            vx.zero_()
+            vy.zero_()
+        _, e, c, status = b.solve(vx, vy, None, tile=(32, 32), k=4, overlap=0, seed=5, **kw)
+        torch.cuda.synchronize()
+        assert np.isfinite(e).all()
+        outs.append((vx.cpu().numpy(), vy.cpu().numpy(), list(e), list(c), list(status)))
+        b.close()
+    assert outs[0][2:] == outs[1][2:]
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])

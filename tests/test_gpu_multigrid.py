@@ -216,3 +216,34 @@ def test_nan_viscosity_is_reported_as_diverged(api):
         ctx.vcycle(vx, vy, None, variant="ras", tile=(32, 32), k=4, overlap=3, inner="f32", tol=1e-8, max_cycles=20)
     assert e.value.status == api.STOKES_ERR_DIVERGED
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [(512, 512), (1024, 768)])
+@pytest.mark.parametrize("after", [dict(variant="rbgs"), dict(variant="jacobi"),
+                                   dict(variant="ras", tile=(32, 32), k=4, overlap=0, seed=5)])
+def test_a_diverged_solve_leaves_no_trace(api, n, after):
+    """A solve whose FP32 V-cycle overflows (omega far too large; sweeps by row
+    streaming, by the pair kernel and by clusters) keeps its hierarchy; the next
+    solve on the context, with a smoother that writes unknowns only, equals that
+    of a fresh context bit for bit."""
+    import torch
+    nx, ny = n
+    prob = inputs.sinker_problem(nx, ny, lx=1.0, ly=ny / nx, eta_in=1e3)
+    kw = dict(nu_max=20, inner="f32", krylov=True, tol=1e-12, max_cycles=3)
+    outs = []
+    for overflow in (False, True):
+        ctx = api.StokesContext(nx, ny, prob.lx, prob.ly, "f64")
+        ctx.set_problem(prob)
+        vx, vy = ctx.field(), ctx.field()
+        if overflow:
+            with pytest.raises(api.StokesError) as e:
+                ctx.vcycle(vx, vy, None, variant="ras", tile=(48, 32), k=8, overlap=7, omega=1e30, **kw)
+            assert e.value.status == api.STOKES_ERR_DIVERGED
+            vx.zero_()
+            vy.zero_()
+        st, e, c = ctx.vcycle(vx, vy, None, **kw, **after)
+        torch.cuda.synchronize()
+        outs.append((ctx.unpack(vx, "vx"), ctx.unpack(vy, "vy"), e, c))
+        ctx.close()
+    assert np.isfinite(outs[0][2]) and outs[0][2:] == outs[1][2:]
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
