@@ -60,6 +60,14 @@ struct Profiler {
     std::vector<cudaEvent_t> pool;
 };
 
+// what the captured V-cycle depends on beside the context's buffers: the
+// parameters and the options that select its kernels (compared by bytes)
+struct GraphKey {
+    stokes_mg_params p;
+    long long wait_limit;
+    int use_tma, pair_mode;
+};
+
 struct stokes_ctx {
     int nx, ny, dtype, pitch, device;
     double lx, ly, hx, hy;
@@ -97,7 +105,7 @@ struct stokes_ctx {
     cudaEvent_t gev[2] = {nullptr, nullptr};
     cudaGraphExec_t gexec = nullptr;
     const void *gz[2] = {nullptr, nullptr}; // where the captured V-cycle leaves z (inner precision, krylov = 1)
-    unsigned char gkey[sizeof(stokes_mg_params)] = {};
+    GraphKey gkey;
     long long gkernels[STOKES_K_COUNT] = {};
 };
 
@@ -405,7 +413,13 @@ int ensure_inner_work(stokes_ctx *c, int dtype)
 // the refinement mode.
 int ensure_graph(stokes_ctx *c, const stokes_mg_params *p)
 {
-    if (c->gexec && std::memcmp(p, c->gkey, sizeof *p) == 0) return STOKES_OK;
+    GraphKey key;
+    std::memset(&key, 0, sizeof key);
+    std::memcpy(&key.p, p, sizeof *p);
+    key.wait_limit = c->wait_limit;
+    key.use_tma = c->use_tma;
+    key.pair_mode = c->pair_mode;
+    if (c->gexec && std::memcmp(&key, &c->gkey, sizeof key) == 0) return STOKES_OK;
     if (p->krylov == 2) {
         const int st = ensure_inner_work(c, p->inner_dtype);
         if (st != STOKES_OK) return st;
@@ -444,7 +458,7 @@ int ensure_graph(stokes_ctx *c, const stokes_mg_params *p)
         c->gexec = nullptr;
         return cuda_fail(ei, "cudaGraphInstantiate");
     }
-    std::memcpy(c->gkey, p, sizeof *p);
+    std::memcpy(&c->gkey, &key, sizeof key);
     for (int k = 0; k < STOKES_K_COUNT; ++k) c->gkernels[k] = hook.k[k];
     return STOKES_OK;
 }

@@ -247,3 +247,43 @@ def test_a_diverged_solve_leaves_no_trace(api, n, after):
         ctx.close()
     assert np.isfinite(outs[0][2]) and outs[0][2:] == outs[1][2:]
     assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
+def test_options_set_between_solves_take_effect(api):
+    """The captured V-cycle follows STOKES_OPT_PAIRED and STOKES_OPT_USE_TMA: after
+    a change a solve launches what a context with that option from the start
+    launches, with the same result; and back."""
+    import torch
+    n = 512
+    prob = inputs.sinker_problem(n, n, eta_in=1e3)
+    kw = dict(variant="ras", tile=(48, 32), k=8, overlap=7, nu_max=20, inner="f32", krylov=True, tol=1e-12,
+              max_cycles=2)
+
+    def solve(ctx):
+        vx, vy = ctx.field(), ctx.field()
+        ctx.profile_reset()
+        ctx.vcycle(vx, vy, None, **kw)
+        torch.cuda.synchronize()
+        return {q: v[0] for q, v in ctx.profile().items()}, ctx.unpack(vx, "vx"), ctx.unpack(vy, "vy")
+
+    def fresh(*options):
+        ctx = api.StokesContext(n, n, 1.0, 1.0, "f64")
+        ctx.set_problem(prob)
+        for o in options:
+            ctx.set_option(*o)
+        solve(ctx)  # builds the hierarchy
+        out = solve(ctx)
+        return ctx, out
+
+    ctx, default = fresh()
+    for opt in ((api.STOKES_OPT_PAIRED, 0), (api.STOKES_OPT_USE_TMA, 0)):
+        other, want = fresh(opt)
+        other.close()
+        assert want[0] != default[0]
+        ctx.set_option(*opt)
+        got = solve(ctx)
+        assert got[0] == want[0]
+        assert np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
+        ctx.set_option(opt[0], 1)
+        assert solve(ctx)[0] == default[0]
+    ctx.close()
