@@ -23,6 +23,7 @@ constexpr int MG_MAX_DENSE = 1024; // unknowns of the coarsest level
 struct MgHierarchy {
     bool stale = true;
     int dtype = -1, levels_req = -1, coarsest_req = -1;
+    long long builds = 0; // times the buffers were given back and allocated anew
     int L = 0;
     MgLevel lv[MG_MAX_LEVELS] = {};
     void *vel = nullptr;  // vx, vy of every level, back to back: one memset zeroes them all
@@ -327,6 +328,8 @@ void mg_destroy(MgHierarchy *h)
     delete h;
 }
 
+long long mg_builds(const MgHierarchy *h) { return h ? h->builds : 0; }
+
 int mg_levels(const MgHierarchy *h) { return h ? h->L : 0; }
 
 int mg_dtype(const MgHierarchy *h) { return h ? h->dtype : -1; }
@@ -350,6 +353,7 @@ int mg_ensure(MgHierarchy **hp, const MgOuter &o, const stokes_mg_params *p, cud
         return STOKES_OK;
     if (cudaStreamSynchronize(s) != cudaSuccess) return STOKES_ERR_CUDA;
     free_all(h);
+    ++h->builds;
     h->stale = true;
     const int st = p->inner_dtype == STOKES_F64 ? build<double>(h, o, p->levels, p->coarsest, s)
                                                 : build<float>(h, o, p->levels, p->coarsest, s);

@@ -39,6 +39,8 @@ void mg_destroy(MgHierarchy *h);
 int mg_ensure(MgHierarchy **h, const MgOuter &o, const stokes_mg_params *params, cudaStream_t s);
 
 // Number of levels of a built hierarchy, and level l of it.
+// how often the buffers have been allocated anew (a captured V-cycle holds their addresses)
+long long mg_builds(const MgHierarchy *h);
 int mg_levels(const MgHierarchy *h);
 const MgLevel &mg_level(const MgHierarchy *h, int l);
 

@@ -61,10 +61,11 @@ struct Profiler {
 };
 
 // what the captured V-cycle depends on beside the context's buffers: the
-// parameters and the options that select its kernels (compared by bytes)
+// parameters, the options that select its kernels and the hierarchy whose
+// buffers it holds (compared by bytes)
 struct GraphKey {
     stokes_mg_params p;
-    long long wait_limit;
+    long long wait_limit, builds;
     int use_tma, pair_mode;
 };
 
@@ -417,6 +418,7 @@ int ensure_graph(stokes_ctx *c, const stokes_mg_params *p)
     std::memset(&key, 0, sizeof key);
     std::memcpy(&key.p, p, sizeof *p);
     key.wait_limit = c->wait_limit;
+    key.builds = mg_builds(c->mg);
     key.use_tma = c->use_tma;
     key.pair_mode = c->pair_mode;
     if (c->gexec && std::memcmp(&key, &c->gkey, sizeof key) == 0) return STOKES_OK;

@@ -287,3 +287,30 @@ def test_options_set_between_solves_take_effect(api):
         ctx.set_option(opt[0], 1)
         assert solve(ctx)[0] == default[0]
     ctx.close()
+
+
+def test_a_refused_hierarchy_leaves_no_captured_cycle(api):
+    """Parameters whose coarsest level is too large are refused after the kept
+    hierarchy has been given back; the first parameters then capture their
+    V-cycle again on the new buffers, with the first result."""
+    n = 256
+    prob = inputs.sinker_problem(n, n, eta_in=1e3)
+    kw = dict(variant="ras", tile=(32, 32), k=4, overlap=3, nu_max=20, inner="f32", krylov=True, tol=1e-12,
+              max_cycles=2)
+    ctx = api.StokesContext(n, n, 1.0, 1.0, "f64")
+    ctx.set_problem(prob)
+    outs = []
+    for _ in range(2):
+        vx, vy = ctx.field(), ctx.field()
+        ctx.vcycle(vx, vy, None, **kw)
+        outs.append((ctx.unpack(vx, "vx"), ctx.unpack(vy, "vy")))
+        # other buffers in the place of those given back
+        other = api.StokesContext(n // 2, n, 1.0, 1.0, "f64")
+        with pytest.raises(api.StokesError) as e:
+            ctx.vcycle(vx, vy, None, **dict(kw, levels=2))
+        assert e.value.status == api.STOKES_ERR_ARG
+        more = api.StokesContext(n, n // 2, 1.0, 1.0, "f64")
+        more.set_problem(inputs.sinker_problem(n, n // 2, ly=0.5, eta_in=1e3))
+        other.close()
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+    ctx.close()
