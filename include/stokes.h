@@ -363,6 +363,30 @@ typedef enum {
 int stokes_tile_kernel_plan(int nx, int ny, int ti, int tj, int overlap, int dtype, int use_tma, int pair_mode,
                             int *kernel, int *threads, size_t *smem_bytes);
 
+/* Which kernels stokes_smooth runs for these parameters on an nx x ny grid, with
+ * the given STOKES_OPT_USE_TMA and STOKES_OPT_PAIRED values.  max_cluster: CTAs
+ * of the largest thread-block cluster to plan for, 0 for what the current
+ * device runs; with a positive value the call reads no device.  Diagnostic only:
+ * it answers for parameters that stokes_smooth accepts.  STOKES_ERR_ARG on
+ * sizes < 2, a bad dtype, variant (STOKES_MIXED among them), pair mode or
+ * schedule, or a NULL pointer. */
+typedef enum {
+    STOKES_PATH_PASSES = 0, /* a pass over the grid per sweep (Jacobi, and RBGS on its own tiles) */
+    STOKES_PATH_TILES = 1,  /* a tile kernel (stokes_tile_kernel_plan), one launch per outer iteration or sweep */
+    STOKES_PATH_STREAM = 2, /* row streaming, several sweeps a pass */
+    STOKES_PATH_CLUSTER = 3 /* all sweeps in one launch of one cluster of CTAs */
+} stokes_smooth_path;
+
+typedef struct {
+    int path;                      /* stokes_smooth_path */
+    int passes;                    /* launches of the sweep kernel */
+    int tile_i, tile_j, k, overlap; /* STOKES_PATH_TILES: the tiles and schedule it runs, else 0 */
+    int cluster;                   /* STOKES_PATH_CLUSTER: CTAs, else 0 */
+} stokes_smooth_plan_info;
+
+int stokes_smooth_plan(int nx, int ny, int dtype, const stokes_smooth_params *params, int use_tma, int pair_mode,
+                       int max_cluster, stokes_smooth_plan_info *plan);
+
 /* Energy residual sums without allocating.  The paper has no counterpart: this
  * entry point exists for callers that cannot call cudaMalloc, for instance
  * code that runs inside a framework's device-memory budget that forbids side

@@ -73,6 +73,10 @@ class stokes3d_smooth_params(ctypes.Structure):
                 ("shifts", ctypes.POINTER(ctypes.c_int32))]
 
 
+class stokes_smooth_plan_info(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int) for n in ("path", "passes", "tile_i", "tile_j", "k", "overlap", "cluster")]
+
+
 _VP, _I, _D = ctypes.c_void_p, ctypes.c_int, ctypes.c_double
 _SIGS = {
     "stokes_create": (_I, [_I, _I, _D, _D, _I, _VP, ctypes.POINTER(_VP)]),
@@ -91,6 +95,8 @@ _SIGS = {
     "stokes_synchronize": (_I, [_VP]),
     "stokes_tile_kernel_plan": (_I, [_I, _I, _I, _I, _I, _I, _I, _I, ctypes.POINTER(_I), ctypes.POINTER(_I),
                                      ctypes.POINTER(ctypes.c_size_t)]),
+    "stokes_smooth_plan": (_I, [_I, _I, _I, ctypes.POINTER(stokes_smooth_params), _I, _I, _I,
+                                ctypes.POINTER(stokes_smooth_plan_info)]),
     "stokes_profile_reset": (_I, [_VP, _I]),
     "stokes_profile_read": (_I, [_VP, _I, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong),
                                  ctypes.POINTER(_D)]),
@@ -287,6 +293,20 @@ def stokes_tile_kernel_plan(nx, ny, tile, overlap, dtype="f32", use_tma=True, pa
                                           int(pair_mode), ctypes.byref(kern), ctypes.byref(thr),
                                           ctypes.byref(smem)), "stokes_tile_kernel_plan")
     return TILE_KERNELS[kern.value], thr.value, smem.value
+
+
+SMOOTH_PATHS = ["passes", "tiles", "stream", "cluster"]
+
+
+def stokes_smooth_plan(nx, ny, params, dtype="f32", use_tma=True, pair_mode=1, max_cluster=0):
+    """The kernels of a smoothing call, as a dict: path (SMOOTH_PATHS), passes,
+    tile, k and overlap of a tile path, cluster (CTAs)."""
+    out = stokes_smooth_plan_info()
+    code = STOKES_F64 if dtype in ("f64", "float64") else STOKES_F32
+    _check(_lib().stokes_smooth_plan(nx, ny, code, ctypes.byref(params), 1 if use_tma else 0, int(pair_mode),
+                                     int(max_cluster), ctypes.byref(out)), "stokes_smooth_plan")
+    return dict(path=SMOOTH_PATHS[out.path], passes=out.passes, tile=(out.tile_i, out.tile_j), k=out.k,
+                overlap=out.overlap, cluster=out.cluster)
 
 
 def stokes_profile_reset(ctx, enable_timing):

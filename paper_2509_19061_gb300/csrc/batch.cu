@@ -200,7 +200,7 @@ int plan_group(Owned &o, const std::vector<GInst<T>> &gi, const RasForm &f, bool
         RasRun r{};
         r.allow_tma = tma;
         r.pair_mode = pair_mode;
-        n_stream = stream_batch_passes(cells, f.sweeps, r);
+        n_stream = stream_passes(cells, f.sweeps, r);
     }
     const int n_outer = (f.sweeps + f.k - 1) / f.k;
     for (int t = 0; t < n_outer; ++t) {

@@ -20,6 +20,7 @@
 // FP64 64^2 415 and 85 us, 32^2 329 and 52; FP32 64^2 66 and 28, 128^2 66 and
 // 40.  A sweep costs 0.45 us at the least, most of it the cluster barrier.
 #include <algorithm>
+#include <atomic>
 
 #include <cooperative_groups.h>
 
@@ -34,6 +35,8 @@ namespace cg = cooperative_groups;
 
 constexpr int CL_MAX_CTAS = 16;
 constexpr int CL_MAX_COLS = 256;
+constexpr int CL_MAX_THREADS = 512;
+constexpr size_t CL_MAX_SMEM = (size_t)200 * 1024;
 
 template <typename T>
 struct ClusterArgs {
@@ -53,7 +56,7 @@ __host__ __device__ constexpr int cl_elems(int cols, int band) { return cl_pitch
 
 // R rows of one column per thread; thread (column, row group)
 template <typename T, int R, bool SQ>
-__global__ void __launch_bounds__(512) k_jacobi_cluster(const __grid_constant__ ClusterArgs<T> a)
+__global__ void __launch_bounds__(CL_MAX_THREADS) k_jacobi_cluster(const __grid_constant__ ClusterArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char cl_raw[];
     cg::cluster_group cluster = cg::this_cluster();
@@ -199,23 +202,24 @@ struct ClusterPlan {
     size_t smem;
 };
 
+// `most`: CTAs of the largest cluster
 template <typename T>
-bool cluster_plan(int nx, int ny, ClusterPlan<T> *p)
+bool cluster_plan(int nx, int ny, int most, ClusterPlan<T> *p)
 {
     if (nx > CL_MAX_COLS || ny < 2) return false;
     // FP64 wants every SM it can get; FP32 CTAs of at least 256 cells, below
     // which the barrier dominates
     const int cells = nx * ny, per = sizeof(T) == 8 ? 32 : 256;
     int c = 1;
-    while (c < CL_MAX_CTAS && c * 2 <= ny / 2 && cells >= c * 2 * per) c *= 2;
+    while (c * 2 <= most && c * 2 <= ny / 2 && cells >= c * 2 * per) c *= 2;
     p->ctas = c;
     p->band = (ny + c - 1) / c;
     p->cols = (nx + 31) / 32 * 32;
     p->rows = 1;
-    while (p->rows < 8 && p->cols * ((p->band + p->rows - 1) / p->rows) > 512) p->rows *= 2;
+    while (p->rows < 8 && p->cols * ((p->band + p->rows - 1) / p->rows) > CL_MAX_THREADS) p->rows *= 2;
     p->threads = p->cols * ((p->band + p->rows - 1) / p->rows);
     p->smem = (size_t)cl_elems(p->cols, p->band) * sizeof(T);
-    return p->threads <= 512 && p->smem <= (size_t)200 * 1024;
+    return p->threads <= CL_MAX_THREADS && p->smem <= CL_MAX_SMEM;
 }
 
 template <typename T, int R>
@@ -224,7 +228,55 @@ void (*pick_cluster(bool square))(ClusterArgs<T>)
     return square ? k_jacobi_cluster<T, R, true> : k_jacobi_cluster<T, R, false>;
 }
 
+// CTAs of the largest cluster that the current device runs of the largest CTA
+// used here (one an SM, so it does not depend on the kernel): 16 where a GPC
+// has that many SMs free for one client, else less; 0 if none.  Asked once per
+// device.
+int cluster_limit()
+{
+    static std::atomic<int> known[16]; // limit + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    const bool cached = dev >= 0 && dev < 16;
+    if (cached)
+        if (const int k = known[dev].load(std::memory_order_relaxed)) return k - 1;
+    const auto kern = k_jacobi_cluster<float, 1, true>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_MAX_SMEM);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    int c = CL_MAX_CTAS;
+    for (; c > 0; c /= 2) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)c);
+        cfg.blockDim = dim3(CL_MAX_THREADS);
+        cfg.dynamicSmemBytes = CL_MAX_SMEM;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)c;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) break;
+    }
+    cudaGetLastError();
+    if (cached) known[dev].store(c + 1, std::memory_order_relaxed);
+    return c;
+}
+
+int most_ctas(const RasRun &run) { return run.max_cluster > 0 ? std::min(run.max_cluster, CL_MAX_CTAS) : cluster_limit(); }
+
 } // namespace
+
+template <typename T>
+int cluster_ctas(int nx, int ny, const RasRun &run)
+{
+    ClusterPlan<T> p;
+    return cluster_plan<T>(nx, ny, most_ctas(run), &p) ? p.ctas : 0;
+}
 
 template <typename T>
 bool cluster_takes(int nx, int ny, int sweeps, const RasRun &run)
@@ -238,15 +290,17 @@ bool cluster_takes(int nx, int ny, int sweeps, const RasRun &run)
     // FP64: 141 us, 85 for as many cells in 64 rows).
     if ((long long)nx * ny > (sizeof(T) == 8 ? 4608 : 16384)) return false;
     ClusterPlan<T> p;
-    return sweeps >= 2 && cluster_plan<T>(nx, ny, &p);
+    if (sweeps < 2) return false;
+    const int most = most_ctas(run); // (no cluster to be had: the tiles)
+    return most > 0 && cluster_plan<T>(nx, ny, most, &p);
 }
 
 template <typename T>
 cudaError_t launch_jacobi_cluster(const GridDesc<T> &g, const Coeffs<T> &c, T omega, int sweeps, T *vx, T *vy,
-                                  cudaStream_t s)
+                                  const RasRun &run, cudaStream_t s)
 {
     ClusterPlan<T> p;
-    if (!c.inv_dx || !c.inv_dy || !cluster_plan<T>(g.nx, g.ny, &p)) return cudaErrorInvalidValue;
+    if (!c.inv_dx || !c.inv_dy || !cluster_plan<T>(g.nx, g.ny, most_ctas(run), &p)) return cudaErrorInvalidValue;
     ClusterArgs<T> a;
     a.g = g;
     a.c = c;
@@ -279,11 +333,13 @@ cudaError_t launch_jacobi_cluster(const GridDesc<T> &g, const Coeffs<T> &c, T om
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
+template int cluster_ctas<float>(int, int, const RasRun &);
+template int cluster_ctas<double>(int, int, const RasRun &);
 template bool cluster_takes<float>(int, int, int, const RasRun &);
 template bool cluster_takes<double>(int, int, int, const RasRun &);
 template cudaError_t launch_jacobi_cluster<float>(const GridDesc<float> &, const Coeffs<float> &, float, int, float *,
-                                                  float *, cudaStream_t);
+                                                  float *, const RasRun &, cudaStream_t);
 template cudaError_t launch_jacobi_cluster<double>(const GridDesc<double> &, const Coeffs<double> &, double, int,
-                                                   double *, double *, cudaStream_t);
+                                                   double *, double *, const RasRun &, cudaStream_t);
 
 } // namespace stokes

@@ -132,6 +132,7 @@ struct RasRun {
     int pair_mode = 1;     // FP32 packed-pair TMA kernel: 0 never, 1 windows of 49-64 columns, 2 any window <= 64
     int *status;           // device word set to 1 when a bounded wait gives up
     long long wait_limit;  // SM cycles a wait may take
+    int max_cluster = 0;   // CTAs of the largest cluster to use; 0: what the device runs
 };
 // One RAS outer iteration: `ksweeps` local Jacobi sweeps on each tile grown by
 // `overlap`, reading (vx, vy), writing the owned unknowns to (ox, oy).
@@ -140,14 +141,15 @@ cudaError_t launch_ras(const GridDesc<T> &g, const Coeffs<T> &c, T omega, const 
                        int overlap, const T *vx, const T *vy, T *ox, T *oy, const RasRun &run, cudaStream_t s);
 // Row-streaming form of a RAS schedule that equals global Jacobi (FP32,
 // stream_kernels.cu): the number of passes that `sweeps` sweeps take (near
-// equal shares of them each), 0 where the tile kernels run it instead, and one
-// pass of `sweeps` sweeps from (vx, vy) to the unknowns of (ox, oy).
-int stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run);
+// equal shares of them each) on a grid, or a batch, of `cells` cells, 0 where the
+// tile kernels run it instead, and one pass of `sweeps` sweeps from (vx, vy) to
+// the unknowns of (ox, oy).
+int stream_passes(long long cells, int sweeps, const RasRun &run);
 cudaError_t launch_ras_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
                               const float *vx, const float *vy, float *ox, float *oy, cudaStream_t s);
 
 // the same in FP64 (stream64_kernels.cu)
-int stream64_passes(const GridDesc<double> &g, int sweeps, const RasRun &run);
+int stream64_passes(int nx, int ny, int sweeps, const RasRun &run);
 cudaError_t launch_ras_stream64(const GridDesc<double> &g, const Coeffs<double> &c, double omega, int sweeps,
                                 const double *vx, const double *vy, double *ox, double *oy, cudaStream_t s);
 
@@ -173,8 +175,6 @@ StreamEntry stream_entry(const GridDesc<float> &g, const Coeffs<float> &c, float
 // Splits the rows of `n` entries into segments for one launch; returns the
 // number of tasks (the sum of strips x segs).
 int stream_split(StreamEntry *e, int n);
-// Passes of a batch over `cells` cells altogether, as stream_passes.
-int stream_batch_passes(long long cells, int sweeps, const RasRun &run);
 // One pass over the tasks of a batch (device tables), all of `sweeps` sweeps
 // and square or not; entries whose live[inst] is 0 are skipped.
 cudaError_t launch_ras_stream_batch(const StreamEntry *tab, const StreamTask *tasks, int ntasks, int sweeps,
@@ -182,17 +182,19 @@ cudaError_t launch_ras_stream_batch(const StreamEntry *tab, const StreamTask *ta
 // Red-black Gauss-Seidel by row streaming (FP32, rbgs_kernels.cu): the passes
 // that `sweeps` sweeps take, 0 where launch_rbgs_sweep runs them instead, and
 // one pass of one or two sweeps.
-int rbgs_stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run);
+int rbgs_stream_passes(int nx, int ny, int sweeps, const RasRun &run);
 cudaError_t launch_rbgs_stream(const GridDesc<float> &g, const Coeffs<float> &c, float omega, int sweeps,
                                const float *vx, const float *vy, float *ox, float *oy, cudaStream_t s);
 // All sweeps of a small grid's damped Jacobi in one launch, in place
-// (cluster_kernels.cu): whether a smoothing of `sweeps` sweeps takes it, and
-// the launch.
+// (cluster_kernels.cu): whether a smoothing of `sweeps` sweeps takes it, on how
+// many CTAs, and the launch.
 template <typename T>
 bool cluster_takes(int nx, int ny, int sweeps, const RasRun &run);
 template <typename T>
+int cluster_ctas(int nx, int ny, const RasRun &run);
+template <typename T>
 cudaError_t launch_jacobi_cluster(const GridDesc<T> &g, const Coeffs<T> &c, T omega, int sweeps, T *vx, T *vy,
-                                  cudaStream_t s);
+                                  const RasRun &run, cudaStream_t s);
 // shared memory a RAS launch needs for this grid, tile and overlap
 size_t ras_smem_bytes(int nx, int ny, int ti, int tj, int overlap, size_t elem);
 // Whether a Jacobi-equivalent smoothing of an nx x ny level runs all its sweeps
@@ -314,8 +316,16 @@ template <typename T>
 int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx, T *sy, const SmoothSpec &p,
                    const RasRun &run, cudaStream_t s, LaunchHook &hook, bool *swapped = nullptr, T *tx = nullptr,
                    T *ty = nullptr, bool zero_walls = false);
-// ping-pong passes of one smoothing call
+// Which kernels a smoothing of an nx x ny grid runs: all sweeps by one cluster
+// of CTAs, `stream` passes of a row-streaming kernel, or else its passes on the
+// tiles of `tiles` (RAS, blocked Jacobi) or on the whole grid.
+struct SmoothPlan {
+    bool cluster;
+    int stream;
+    SmoothSpec tiles;
+    int passes; // ping-pong passes, at least 1 if there are sweeps
+};
 template <typename T>
-int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run);
+SmoothPlan smooth_plan(int nx, int ny, const SmoothSpec &p, const RasRun &run);
 
 } // namespace stokes

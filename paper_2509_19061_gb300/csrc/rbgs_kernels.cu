@@ -255,13 +255,13 @@ __global__ void __launch_bounds__(RB_MAX * 32, RB_CTAS) k_rbgs_stream(const __gr
 
 } // namespace
 
-int rbgs_stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run)
+int rbgs_stream_passes(int nx, int ny, int sweeps, const RasRun &run)
 {
     // One sweep, or two on the smaller grids, gain less than the copy back that an
     // odd pass count costs: 8192^2 one sweep 1014 us, 962 by tiles; two at 640^2
     // 28.4 and 26.4, at 1024^2 37.9 and 39.7.
     const long long least = sweeps == 2 ? 2 * RB_MIN_CELLS : RB_MIN_CELLS;
-    if (!run.allow_tma || run.pair_mode != 1 || sweeps < 2 || (long long)g.nx * g.ny < least) return 0;
+    if (!run.allow_tma || run.pair_mode != 1 || sweeps < 2 || (long long)nx * ny < least) return 0;
     return (sweeps + RB_MAX - 1) / RB_MAX;
 }
 

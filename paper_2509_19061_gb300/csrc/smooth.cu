@@ -14,25 +14,19 @@ bool any_traversal(const SmoothSpec &p)
     return (p.variant == STOKES_RAS && p.overlap >= p.k - 1) || p.variant == STOKES_JACOBI_FUSED;
 }
 
-template <typename T>
-bool takes_cluster(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
-{
-    return any_traversal(p) && cluster_takes<T>(g.nx, g.ny, p.sweeps, run);
-}
-
 // passes of a row-streaming kernel for this smoothing, 0 if none takes it: red-
 // black Gauss-Seidel's own; else a RAS schedule with overlap >= k - 1 is global
 // Jacobi in any traversal, and fused Jacobi's sweeps need not each cross the
 // grid before the next begins (20 sweeps of 4001 x 2999: 408 us, 1822 us as 20
 // passes of k_jacobi_rows).  Separate-pass and blocked Jacobi keep their passes.
 template <typename T>
-int stream_passes_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
+int stream_passes_of(int nx, int ny, const SmoothSpec &p, const RasRun &run)
 {
     if constexpr (sizeof(T) == 4)
-        if (p.variant == STOKES_RBGS) return rbgs_stream_passes(g, p.sweeps, run);
+        if (p.variant == STOKES_RBGS) return rbgs_stream_passes(nx, ny, p.sweeps, run);
     if (!any_traversal(p)) return 0;
-    if constexpr (sizeof(T) == 4) return stream_passes(g, p.sweeps, run);
-    else return stream64_passes(g, p.sweeps, run);
+    if constexpr (sizeof(T) == 4) return stream_passes((long long)nx * ny, p.sweeps, run);
+    else return stream64_passes(nx, ny, p.sweeps, run);
 }
 
 // The tiles of an FP32 RAS schedule that equals global Jacobi, on grids between
@@ -47,10 +41,10 @@ int stream_passes_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &ru
 // 25.0 ms, now 24.1; 8 CG cycles of 1024^2 (48 x 32, k = 8) 7.28 and 7.11.
 constexpr long long FREE_MAX_CELLS = 600000; // where the row streaming starts
 template <typename T>
-SmoothSpec tiles_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
+SmoothSpec tiles_of(int nx, int ny, const SmoothSpec &p, const RasRun &run)
 {
     if (sizeof(T) != 4 || p.variant != STOKES_RAS || p.sweeps < 1 || !any_traversal(p) || !run.allow_tma ||
-        run.pair_mode != 1 || p.k > 8 || g.nx < 64 || g.ny < 40 || (long long)g.nx * g.ny >= FREE_MAX_CELLS)
+        run.pair_mode != 1 || p.k > 8 || nx < 64 || ny < 40 || (long long)nx * ny >= FREE_MAX_CELLS)
         return p;
     SmoothSpec q = p;
     const int passes = (p.sweeps + 7) / 8;
@@ -61,7 +55,7 @@ SmoothSpec tiles_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run
     long long best = 0;
     for (int rows : {40, 50, 65, 80}) {
         const int tj = rows - 2 * q.k;
-        const long long tiles = (long long)((g.nx + q.ti - 1) / q.ti) * ((g.ny + tj - 1) / tj);
+        const long long tiles = (long long)((nx + q.ti - 1) / q.ti) * ((ny + tj - 1) / tj);
         const long long cost = (tiles + 151) / 152 * (32 + rows);
         if (best == 0 || cost < best) {
             best = cost;
@@ -73,17 +67,23 @@ SmoothSpec tiles_of(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run
 
 } // namespace
 
-// number of ping-pong passes of a smoothing (one per sweep; one per outer
-// iteration of RAS, or per pass of the row-streaming kernel)
+// (passes: one per sweep, per outer iteration of RAS or per pass of a
+// row-streaming kernel)
 template <typename T>
-int smooth_passes(const GridDesc<T> &g, const SmoothSpec &p, const RasRun &run)
+SmoothPlan smooth_plan(int nx, int ny, const SmoothSpec &p, const RasRun &run)
 {
-    if (p.sweeps <= 0) return 0;
-    if (takes_cluster(g, p, run)) return 1;
-    if (const int n = stream_passes_of(g, p, run)) return n;
-    const int k = tiles_of(g, p, run).k;
-    if (p.variant == STOKES_RAS) return (p.sweeps + k - 1) / k;
-    return p.sweeps;
+    SmoothPlan n{false, 0, tiles_of<T>(nx, ny, p, run), p.sweeps};
+    if (p.sweeps <= 0) {
+        n.passes = 0;
+    } else if (any_traversal(p) && cluster_takes<T>(nx, ny, p.sweeps, run)) {
+        n.cluster = true;
+        n.passes = 1;
+    } else if ((n.stream = stream_passes_of<T>(nx, ny, p, run)) > 0) {
+        n.passes = n.stream;
+    } else if (p.variant == STOKES_RAS) {
+        n.passes = (p.sweeps + n.tiles.k - 1) / n.tiles.k;
+    }
+    return n;
 }
 
 template <typename T>
@@ -100,10 +100,10 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
         if (st != STOKES_OK) return st;                                                                            \
     } while (0)
     if (p.sweeps == 0) return STOKES_OK;
-    const SmoothSpec q = tiles_of(g, p, run); // what the tile launches run
-    const int n_outer = p.variant == STOKES_RAS ? (p.sweeps + q.k - 1) / q.k : 0;
-    const bool cluster = takes_cluster(g, p, run);
-    const int n_stream = stream_passes_of(g, p, run);
+    const SmoothPlan plan = smooth_plan<T>(g.nx, g.ny, p, run);
+    const SmoothSpec &q = plan.tiles; // what the tile launches run
+    const int n_pass = plan.passes, n_stream = plan.stream;
+    const bool cluster = plan.cluster;
     const int kind = p.variant == STOKES_RAS    ? STOKES_K_RAS
                      : p.variant == STOKES_RBGS ? STOKES_K_RBGS
                                                 : STOKES_K_JACOBI;
@@ -113,7 +113,7 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
             if (p.shifts[2 * t] < 0 || p.shifts[2 * t] >= p.ti || p.shifts[2 * t + 1] < 0 || p.shifts[2 * t + 1] >= p.tj)
                 return STOKES_ERR_ARG;
     if (cluster) {
-        LAUNCH(kind, 1, launch_jacobi_cluster<T>(g, k, omega, p.sweeps, vx, vy, s));
+        LAUNCH(kind, 1, launch_jacobi_cluster<T>(g, k, omega, p.sweeps, vx, vy, run, s));
         return STOKES_OK;
     }
     // ping-pong between (vx, vy) and the scratch pair; the scratch walls take
@@ -121,7 +121,6 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     // and an odd number n >= 3 of passes, pass 1 goes from (vx, vy) to (sx, sy),
     // passes 2 .. n-1 alternate between the two scratch pairs and pass n
     // writes (vx, vy): the result lands in place without a copy back.
-    const int n_pass = smooth_passes(g, p, run);
     const bool three = tx && ty && !swapped && n_pass >= 3 && (n_pass & 1);
     T *ax = vx, *ay = vy, *bx = sx, *by = sy;
     if (!zero_walls) LAUNCH(STOKES_K_COPY, 1, launch_copy_walls<T>(g, vx, vy, sx, sy, s));
@@ -157,8 +156,8 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
             advance();
         }
     } else if (p.variant == STOKES_RAS) {
-        for (int t = 0; t < n_outer; ++t) {
-            const int ks = (t == n_outer - 1) ? q.sweeps - (n_outer - 1) * q.k : q.k;
+        for (int t = 0; t < n_pass; ++t) {
+            const int ks = (t == n_pass - 1) ? q.sweeps - (n_pass - 1) * q.k : q.k;
             int si = 0, sj = 0;
             if (q.shift_mode == STOKES_SHIFT_SPLITMIX) {
                 si = (int)(splitmix64(q.seed, 2u * (uint64_t)t) % (uint64_t)q.ti);
@@ -198,8 +197,8 @@ int smooth_buffers(const GridDesc<T> &g, const Coeffs<T> &k, T *vx, T *vy, T *sx
     return STOKES_OK;
 }
 
-template int smooth_passes<float>(const GridDesc<float> &, const SmoothSpec &, const RasRun &);
-template int smooth_passes<double>(const GridDesc<double> &, const SmoothSpec &, const RasRun &);
+template SmoothPlan smooth_plan<float>(int, int, const SmoothSpec &, const RasRun &);
+template SmoothPlan smooth_plan<double>(int, int, const SmoothSpec &, const RasRun &);
 template int smooth_buffers<float>(const GridDesc<float> &, const Coeffs<float> &, float *, float *, float *,
                                    float *, const SmoothSpec &, const RasRun &, cudaStream_t, LaunchHook &, bool *,
                                    float *, float *, bool);

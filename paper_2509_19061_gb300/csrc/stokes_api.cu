@@ -276,7 +276,7 @@ int smooth_impl(stokes_ctx *c, T *vx, T *vy, const stokes_smooth_params *p, int 
         k.by = (const T *)c->fy;
     }
     const SmoothSpec spec = spec_of(p, ti, tj);
-    const int n_pass = smooth_passes(grid_of<T>(c), spec, run_opts(c));
+    const int n_pass = smooth_plan<T>(c->nx, c->ny, spec, run_opts(c)).passes;
     if (n_pass >= 3 && (n_pass & 1) && !c->sx2) { // second scratch pair: odd pass counts end in place
         // A schedule whose own outer iterations would not need the pair (the
         // row-streaming kernel's passes do) ends with a copy instead where it
@@ -1128,6 +1128,38 @@ int stokes_tile_kernel_plan(int nx, int ny, int ti, int tj, int overlap, int dty
     if (kernel) *kernel = kind;
     if (threads) *threads = thr;
     if (smem_bytes) *smem_bytes = smem;
+    return STOKES_OK;
+}
+
+int stokes_smooth_plan(int nx, int ny, int dtype, const stokes_smooth_params *p, int use_tma, int pair_mode,
+                       int max_cluster, stokes_smooth_plan_info *out)
+{
+    if (!p || !out || nx < 2 || ny < 2 || (dtype != STOKES_F32 && dtype != STOKES_F64) || pair_mode < 0 ||
+        pair_mode > 2 || max_cluster < 0 || p->sweeps < 0 || p->variant < STOKES_JACOBI || p->variant > STOKES_RAS ||
+        (p->variant == STOKES_RAS && (p->k < 1 || p->overlap < 0)))
+        return STOKES_ERR_ARG;
+    RasRun run{};
+    run.allow_tma = use_tma != 0;
+    run.pair_mode = pair_mode;
+    run.max_cluster = max_cluster;
+    const SmoothSpec spec = spec_of(p, p->tile_i > 0 ? p->tile_i : 32, p->tile_j > 0 ? p->tile_j : 32);
+    const bool f64 = dtype == STOKES_F64;
+    const SmoothPlan n = f64 ? smooth_plan<double>(nx, ny, spec, run) : smooth_plan<float>(nx, ny, spec, run);
+    *out = stokes_smooth_plan_info{};
+    out->passes = n.passes;
+    if (n.cluster) {
+        out->path = STOKES_PATH_CLUSTER;
+        out->cluster = f64 ? cluster_ctas<double>(nx, ny, run) : cluster_ctas<float>(nx, ny, run);
+    } else if (n.stream > 0) {
+        out->path = STOKES_PATH_STREAM;
+    } else if (p->variant == STOKES_RAS || p->variant == STOKES_JACOBI_BLOCKED) {
+        const bool ras = p->variant == STOKES_RAS;
+        out->path = STOKES_PATH_TILES;
+        out->tile_i = n.tiles.ti;
+        out->tile_j = n.tiles.tj;
+        out->k = ras ? n.tiles.k : 1;
+        out->overlap = ras ? n.tiles.overlap : 0;
+    }
     return STOKES_OK;
 }
 

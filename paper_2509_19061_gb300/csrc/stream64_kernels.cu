@@ -196,11 +196,11 @@ __global__ void __launch_bounds__(S8_MAX * 32, 4) k_stream64(const __grid_consta
 
 } // namespace
 
-int stream64_passes(const GridDesc<double> &g, int sweeps, const RasRun &run)
+int stream64_passes(int nx, int ny, int sweeps, const RasRun &run)
 {
     if (!run.allow_tma || run.pair_mode != 1 || sweeps < 2) return 0;
     // (40 sweeps: 256^2 377 us, 337 on 24 x 24 tiles; 384^2 470 and 544)
-    if ((long long)g.nx * g.ny < S8_MIN_CELLS) return 0;
+    if ((long long)nx * ny < S8_MIN_CELLS) return 0;
     return (sweeps + S8_MAX - 1) / S8_MAX;
 }
 

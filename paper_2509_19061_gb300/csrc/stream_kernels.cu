@@ -337,12 +337,7 @@ int stream_wave()
 
 } // namespace
 
-int stream_passes(const GridDesc<float> &g, int sweeps, const RasRun &run)
-{
-    return stream_batch_passes((long long)g.nx * g.ny, sweeps, run);
-}
-
-int stream_batch_passes(long long cells, int sweeps, const RasRun &run)
+int stream_passes(long long cells, int sweeps, const RasRun &run)
 {
     if (!run.allow_tma || run.pair_mode != 1 || sweeps < ST_MIN_SWEEPS) return 0;
     // Below this a segment's 2 n extra rows outweigh the tiles' halo: 40 sweeps

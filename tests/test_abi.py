@@ -109,3 +109,54 @@ def test_batched_workload_recipe():
     assert all(s.radius + 0.3 > 0 and 0.05 <= s.radius <= 0.2 and 0.3 <= s.cx <= 0.7 for s in a)
     cells = np.array([n * n for n in ns], dtype=np.float64)
     assert 1.0e5 < cells.mean() < 3.0e5
+
+
+@pytest.mark.parametrize("dtype,nx,ny", [("f64", 64, 64), ("f64", 2, 2), ("f64", 250, 18), ("f32", 128, 128),
+                                         ("f32", 33, 31), ("f32", 256, 9), ("f32", 31, 500)])
+def test_small_grids_fit_the_clusters_that_a_device_runs(lib, dtype, nx, ny):
+    """A schedule that one cluster of CTAs runs is planned for the largest cluster
+    that the device has room for, down to one CTA, and goes back to the tiles
+    where that does not hold the grid; no device is read."""
+    from paper_2509_19061_gb300 import api
+    ras = api.smooth_params("ras", sweeps=10, tile=(16, 16), k=4, overlap=3)
+    was = None
+    for most in (1, 2, 4, 8, 16):
+        plan = api.stokes_smooth_plan(nx, ny, ras, dtype, max_cluster=most)
+        if plan["path"] == "cluster":
+            assert 1 <= plan["cluster"] <= most and plan["passes"] == 1
+            assert was in (None, "tiles", "cluster")
+        else:
+            assert plan["path"] == "tiles" and was != "cluster"
+        was = plan["path"]
+    assert was == "cluster"
+
+
+def test_smooth_plan_without_device(lib):
+    """What stokes_smooth runs, by variant, size, dtype and option."""
+    from paper_2509_19061_gb300 import api
+
+    def plan(n, dtype="f32", m=None, use_tma=True, pair_mode=1, **kw):
+        return api.stokes_smooth_plan(n, m or n, api.smooth_params(**kw), dtype, use_tma, pair_mode, 16)
+
+    exact = dict(variant="ras", sweeps=20, tile=(32, 32), k=4, overlap=3)
+    assert plan(8192, **exact) == dict(path="stream", passes=3, tile=(0, 0), k=0, overlap=0, cluster=0)
+    assert plan(1024, "f64", **exact)["path"] == "stream" and plan(1024, "f64", **exact)["passes"] == 5
+    assert plan(8192, pair_mode=2, **exact) == dict(path="tiles", passes=5, tile=(32, 32), k=4, overlap=3, cluster=0)
+    assert plan(8192, use_tma=False, **exact)["path"] == "tiles"
+    mid = plan(512, **exact)
+    assert mid["path"] == "tiles" and mid["tile"][0] == 64 - 2 * mid["k"] and mid["overlap"] == mid["k"] - 1
+    assert plan(128, **exact)["path"] == "cluster"
+    assert plan(8192, **dict(exact, overlap=0))["tile"] == (32, 32)
+    assert plan(2000, variant="rbgs", sweeps=5) == dict(path="stream", passes=3, tile=(0, 0), k=0, overlap=0, cluster=0)
+    assert plan(2000, variant="rbgs", sweeps=1)["path"] == "passes"
+    assert plan(2000, variant="jacobi", sweeps=7) == dict(path="passes", passes=7, tile=(0, 0), k=0, overlap=0, cluster=0)
+    assert plan(2000, variant="blocked", sweeps=7, tile=(24, 16))["tile"] == (24, 16)
+    assert plan(64, **dict(exact, sweeps=0))["passes"] == 0
+    for bad in (dict(variant="mixed"), dict(exact, k=0, overlap=0), dict(exact, pair_mode=3), dict(exact, dtype=7)):
+        kw = dict(bad)
+        with pytest.raises(api.StokesError):
+            if kw.pop("dtype", None) == 7:
+                st = api._lib().stokes_smooth_plan(8, 8, 7, ctypes.byref(api.smooth_params(**kw)), 1, 1, 16,
+                                                   ctypes.byref(api.stokes_smooth_plan_info()))
+                raise api.StokesError(st, "dtype")
+            plan(64, **kw)
