@@ -48,8 +48,13 @@ FLOPS_PER_CELL_SWEEP = 24
 # per SM, an FMA counting 2 flops; FP64 at its nominal 1.25 TFLOP/s
 NOMINAL_FP32_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 NOMINAL_FP64_TFLOPS = 1.25
+# sources of each sweep kernel (the tile kernels otherwise), for the profiles taken on them
 RAS_SOURCES = ["paper_2509_19061_gb300/csrc/ras_kernels.cu", "paper_2509_19061_gb300/csrc/stencil.cuh"]
-STREAM_SOURCES = ["paper_2509_19061_gb300/csrc/stream_kernels.cu", "paper_2509_19061_gb300/csrc/f32x2.cuh"]
+KERNEL_SOURCES = {
+    "k_ras_stream": ["paper_2509_19061_gb300/csrc/stream_kernels.cu", "paper_2509_19061_gb300/csrc/f32x2.cuh"],
+    "k_stream64": ["paper_2509_19061_gb300/csrc/stream64_kernels.cu", "paper_2509_19061_gb300/csrc/stencil.cuh"],
+    "k_jacobi_cluster": ["paper_2509_19061_gb300/csrc/cluster_kernels.cu", "paper_2509_19061_gb300/csrc/stencil.cuh"],
+}
 
 
 def parse():
@@ -322,12 +327,19 @@ def workload_config(args):
 TILE_KERNEL_NAMES = {"pair": "k_ras_pair", "tma": "k_ras_tma", "global": "k_ras_reg", "shared": "k_ras"}
 
 
-def tile_kernel_name(api, n, tile, k, overlap, dt_name):
-    """Name of the kernel the library picks for this schedule: row streaming
-    where it equals global Jacobi on a large grid, else a tile kernel."""
-    if overlap >= k - 1 and n * n >= (600000 if dt_name == "f32" else 100000):
-        return "k_ras_stream" if dt_name == "f32" else "k_ras_stream64"
-    return TILE_KERNEL_NAMES[api.stokes_tile_kernel_plan(n, n, tuple(tile), overlap, dt_name)[0]]
+def sweep_kernel_name(api, n, dt_name, max_cluster=0, **smooth):
+    """Name of the kernel that the library's smoothing of an n x n grid runs
+    (what stokes_smooth_plan says; a pass per sweep has none here)."""
+    plan = api.stokes_smooth_plan(n, n, api.smooth_params(**smooth), dt_name, max_cluster=max_cluster)
+    if plan["path"] == "cluster":
+        return "k_jacobi_cluster"
+    if plan["path"] == "stream":
+        if smooth["variant"] == "rbgs":
+            return "k_rbgs_stream"
+        return "k_ras_stream" if dt_name == "f32" else "k_stream64"
+    if plan["path"] == "tiles":
+        return TILE_KERNEL_NAMES[api.stokes_tile_kernel_plan(n, n, plan["tile"], plan["overlap"], dt_name)[0]]
+    return None
 
 
 def median_ci(xs):
@@ -432,7 +444,8 @@ def run_ours(args):
     # once: 8 words per cell per launch), and the effective bytes of the
     # paper's yardstick (8 words per cell per sweep, which exceeds the HBM
     # peak when k > 1 because the window stays on chip for k sweeps).
-    kernel = tile_kernel_name(api, n, args.tile, k, o, dt_name)
+    kernel = sweep_kernel_name(api, n, dt_name, variant="ras", sweeps=args.sweeps, tile=tuple(args.tile), k=k,
+                               overlap=o)
     sweeps_per_launch = args.sweeps * args.steps / max(ras_groups, 1)
     min_bytes = WORDS_PER_CELL_SWEEP * esize * cells
     eff_bytes = min_bytes * sweeps_per_launch
@@ -440,7 +453,7 @@ def run_ours(args):
     avg_s = avg_ms / 1e3
     peak, peak_kind = measured_peaks()
     key = "ras_%s_%d_t%dx%d_k%d_o%d" % (dt_name, n, args.tile[0], args.tile[1], k, o)
-    sources = source_hash(STREAM_SOURCES if kernel == "k_ras_stream" else RAS_SOURCES)
+    sources = source_hash(KERNEL_SOURCES.get(kernel, RAS_SOURCES))
     traffic = ncu_traffic(key, sources)
     limiter = (ncu_entry(key, sources) or {}).get("limiter")
     flops = FLOPS_PER_CELL_SWEEP * cells * sweeps_per_launch
@@ -993,8 +1006,7 @@ def variant_table(args, api, prob):
         out[label] = {"gcell_updates_per_s": cu / 1e9, "effective_gbs": gbs, "frac": gbs / peak,
                       "sweeps": kw["sweeps"], "ms_per_call": ms}
         if kw["variant"] in ("ras", "blocked"):
-            # (blocked Jacobi always runs the tile kernel)
-            out[label]["kernel"] = tile_kernel_name(api, n, kw["tile"], kw.get("k", 2), kw.get("overlap", 0), dt_name)
+            out[label]["kernel"] = sweep_kernel_name(api, n, dt_name, **kw)
     for c, _, _ in ctxs.values():
         c.close()
     return out

@@ -1,5 +1,7 @@
 """Host-side arithmetic of bench.py (CPU): the energy-norm weights the
 benchmark uses to state the FP32 error equal -diag(M) of the oracle."""
+import os
+
 import numpy as np
 
 import bench
@@ -16,3 +18,24 @@ def test_energy_weights_are_minus_diag_m():
         assert wx.shape == dx.shape and wy.shape == dy.shape
         assert np.allclose(wx, -dx, rtol=1e-14, atol=0.0)
         assert np.allclose(wy, -dy, rtol=1e-14, atol=0.0)
+
+
+def test_the_named_kernel_is_the_one_that_runs():
+    """The kernel a benchmark row names is what the library's plan says, over
+    sizes, precisions, variants and sweep counts, and its profile is tied to that
+    kernel's own sources."""
+    from paper_2509_19061_gb300 import api, build
+    build.build()
+
+    def name(n, dt, **kw):
+        return bench.sweep_kernel_name(api, n, dt, max_cluster=16, **kw)
+
+    exact = dict(variant="ras", tile=(32, 32), k=4, overlap=3)
+    assert name(8192, "f32", sweeps=100, **exact) == "k_ras_stream"
+    assert name(1024, "f64", sweeps=100, **exact) == "k_stream64"
+    assert name(64, "f64", sweeps=10, **exact) == name(128, "f32", sweeps=10, **exact) == "k_jacobi_cluster"
+    assert name(2000, "f32", variant="rbgs", sweeps=20) == "k_rbgs_stream"
+    assert name(2000, "f64", variant="rbgs", sweeps=20) is None
+    for kernel, paths in bench.KERNEL_SOURCES.items():
+        text = "".join(open(os.path.join(bench.ROOT, p)).read() for p in paths)
+        assert kernel + "(" in text, kernel
