@@ -69,7 +69,9 @@ def parse():
     ap.add_argument("--tile", type=int, nargs=2, default=[48, 64])
     ap.add_argument("--k", type=int, default=8)
     ap.add_argument("--overlap", type=int, default=None)
-    ap.add_argument("--no-extras", action="store_true", help="skip the variant table, e2e and CPU baseline")
+    ap.add_argument("--no-extras", action="store_true", help="skip the extra legs, e2e and CPU baseline")
+    ap.add_argument("--tables", default=os.path.join("_build", "bench_tables.json"),
+                    help="file for the whole result with the tables of the extra legs")
     ap.add_argument("--cpu-seconds", type=float, default=12.0, help="target CPU time of the oracle sample")
     ap.add_argument("--solve-n", type=int, default=4096, help="grid of the time-to-1e-8 solve")
     ap.add_argument("--batch", type=int, default=256, help="instances of the batched workload (0: skip)")
@@ -373,6 +375,31 @@ def job_value(world, cells, sweeps, steps, ms_total):
     return world * cells * sweeps * steps / (ms_total / 1e3) / 1e9
 
 
+# the extra legs, whole in the tables file; the printed line has their headline figures
+TABLES = ("fp32_vs_fp64", "variants", "c2_f64_1024", "time_to_1e-8", "batched", "autotune", "uzawa_stokes",
+          "smoother_robustness", "smooth3d", "global_smoothers", "slabs", "cpu_baseline")
+ROOFLINE = ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "kernel_avg_ms", "kernel_share",
+            "sweeps_per_launch")
+
+
+def short_line(line, tables):
+    """The line that is printed: every key of `line` but the extra legs' tables
+    and the roofline's notes, which stand in the file `tables` (a line of all of
+    them is some 23 KB, and a reader that keeps the last few KB of the output
+    gets no line at all)."""
+    out = {k: v for k, v in line.items() if k not in TABLES}
+    if "roofline" in out:
+        out["roofline"] = {k: out["roofline"].get(k) for k in ROOFLINE}
+    solve, cpu = line.get("time_to_1e-8"), line.get("cpu_baseline")
+    if solve:
+        out["time_to_1e-8"] = {"workload": solve["workload"], "unit": "s", "f32_inner": solve["f32_inner"]["seconds"],
+                               "f64_inner": solve["f64_inner"]["seconds"]}
+    if cpu:
+        out["cpu_baseline"] = {k: cpu.get(k) for k in ("value", "unit", "cores", "kind")}
+    out["tables"] = tables
+    return out
+
+
 # ---------------------------------------------------------------------------
 # our arm
 # ---------------------------------------------------------------------------
@@ -523,7 +550,10 @@ def run_ours(args):
         line["cpu_baseline"]["vcycle_solve"] = cpu_vcycle_solve(api)
     ctx.close()
     if rank == 0:
-        print(json.dumps(line))
+        os.makedirs(os.path.dirname(os.path.abspath(args.tables)), exist_ok=True)
+        with open(args.tables, "w") as f:
+            json.dump(line, f, indent=1)
+        print(json.dumps(short_line(line, args.tables)))
     if world > 1:
         dist.destroy_process_group()
     return 0

@@ -39,3 +39,23 @@ def test_the_named_kernel_is_the_one_that_runs():
     for kernel, paths in bench.KERNEL_SOURCES.items():
         text = "".join(open(os.path.join(bench.ROOT, p)).read() for p in paths)
         assert kernel + "(" in text, kernel
+
+
+def test_the_printed_line_is_short():
+    """The line keeps every figure of the run itself; the extra legs' tables stay
+    out of it, so that it fits the last few KB of the output."""
+    import json
+    run = dict(metric="m", value=1110.123456789012, unit="u", n_gpus=1, steps=20, warmup=5, ms_per_step=6.123456789,
+               higher_is_better=True, scaling="weak", vs_baseline=None, dtype="f32", data="synthetic",
+               config={"workload": "w" * 60, "tile": [48, 64], "step": "s" * 60, "l2": "l" * 80}, gpu_launches=1,
+               clocks={"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": []}, step_ms={"median": 6.1, "ci95": [6, 7]},
+               energy_residual_after_step=0.5, e2e={"value": 700.0, "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 2})
+    line = dict(run, roofline=dict({k: 1.0 for k in bench.ROOFLINE}, traffic_note="n" * 300))
+    line.update({k: {"row %d" % i: {"ms_per_call": 1.0} for i in range(60)} for k in bench.TABLES})
+    line["time_to_1e-8"].update(workload="w", f32_inner={"seconds": 0.05}, f64_inner={"seconds": 0.4})
+    line["cpu_baseline"].update(value=0.02, unit="u", cores=1, kind="oracle")
+    out = bench.short_line(line, "tables.json")
+    assert all(out[k] == v for k, v in run.items())
+    assert out["roofline"] == {k: 1.0 for k in bench.ROOFLINE}
+    assert out["time_to_1e-8"]["f32_inner"] == 0.05 and out["cpu_baseline"]["value"] == 0.02
+    assert len(json.dumps(line)) > 20000 and len(json.dumps(out)) < 2500
