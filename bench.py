@@ -550,9 +550,12 @@ def run_ours(args):
         line["cpu_baseline"]["vcycle_solve"] = cpu_vcycle_solve(api)
     ctx.close()
     if rank == 0:
-        os.makedirs(os.path.dirname(os.path.abspath(args.tables)), exist_ok=True)
-        with open(args.tables, "w") as f:
-            json.dump(line, f, indent=1)
+        try:
+            os.makedirs(os.path.dirname(os.path.abspath(args.tables)), exist_ok=True)
+            with open(args.tables, "w") as f:
+                json.dump(line, f, indent=1)
+        except OSError as e:
+            sys.stderr.write("tables not written: %s\n" % e)
         print(json.dumps(short_line(line, args.tables)))
     if world > 1:
         dist.destroy_process_group()
