@@ -866,3 +866,73 @@ def test_row_streaming_keeps_the_walls_of_an_overflowing_field(api, nx, ny, squa
             fin = np.isfinite(a)
             assert not fin.all() and np.array_equal(fin, np.isfinite(b))
             assert np.array_equal(a[fin], b[fin])
+
+
+@pytest.mark.parametrize("nx,ny,sweeps,square", [
+    (1121, 400, 3, True), (1120, 801, 2, False), (4, 210000, 2, False), (210000, 4, 2, True), (960, 450, 5, False),
+])
+def test_rbgs_streams_two_sweeps_a_pass(api, nx, ny, sweeps, square):
+    """Sizes and sweep counts at which red-black Gauss-Seidel does stream (the
+    launch counts say so): one pass of two sweeps with its copy back, an odd last
+    sweep, grids of four columns and rows; value for value the tile kernel's."""
+    prob = rand_problem(nx, ny, 98, lx=1.0, ly=ny / nx if square else 0.7)
+    vx, vy = inputs.random_velocity(nx, ny, 99, 0.1)
+    vx[:, 0], vx[:, nx], vy[0], vy[ny] = 0.3, -0.2, 0.1, 0.4
+    outs = []
+    for pair, launches in ((0, sweeps), (1, (sweeps + 1) // 2)):
+        r = Run(api, prob, "f32", (vx, vy))
+        r.ctx.set_option(api.STOKES_OPT_PAIRED, pair)
+        r.ctx.profile_reset()
+        r.smooth(variant="rbgs", sweeps=sweeps)
+        outs.append(r.v())
+        assert r.ctx.profile()["rbgs"][0] == launches
+        r.ctx.close()
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("tile,k,o", [((48, 64), 8, 7), ((56, 32), 4, 3), ((48, 32), 3, 2)])
+@pytest.mark.parametrize("nx,ny", [(300, 200), (1000, 650)])
+def test_pair_kernel_square_cells_on_the_given_tiles(api, nx, ny, tile, k, o):
+    """Exact schedules kept on the given tiles (STOKES_OPT_PAIRED = 2; by default
+    they run on chosen tiles or by row streaming): the pair kernel's square-cell
+    form at window heights of 40 and 80 rows, value for value the one-column
+    kernel's and fused Jacobi's, in as many launches as the schedule has outer
+    iterations."""
+    prob = rand_problem(nx, ny, 47, lx=nx / 200.0, ly=ny / 200.0)
+    assert prob.lx / nx == prob.ly / ny
+    assert api.stokes_tile_kernel_plan(nx, ny, tile, o, "f32", pair_mode=2)[0] == "pair"
+    v0 = inputs.random_velocity(nx, ny, 48, 0.1)
+    sweeps, outs = 2 * k + 3, []
+    for pair, variant in ((2, "ras"), (0, "ras"), (1, "fused")):
+        r = Run(api, prob, "f32", v0)
+        r.ctx.set_option(api.STOKES_OPT_PAIRED, pair)
+        r.ctx.profile_reset()
+        r.smooth(variant=variant, sweeps=sweeps, tile=tile, k=k, overlap=o, seed=79)
+        if variant == "ras":
+            assert r.ctx.profile()["ras"][0] == (sweeps + k - 1) // k
+        outs.append(r.v())
+        r.ctx.close()
+        assert np.array_equal(outs[0][0], outs[-1][0]) and np.array_equal(outs[0][1], outs[-1][1])
+
+
+@pytest.mark.parametrize("dtype,tile,k,o", [("f32", (48, 64), 8, 7), ("f32", (32, 32), 4, 3), ("f64", (32, 32), 4, 3)])
+def test_benchmark_sequence_on_tiles_equals_row_streaming(api, dtype, tile, k, o):
+    """The benchmark's 100 sweeps of the 1024^2 layered sinker on the given tiles
+    (STOKES_OPT_USE_TMA with STOKES_OPT_PAIRED = 2 or 0: the pair and the
+    one-column kernels; 13 or 25 launches) and by row streaming: the same
+    values."""
+    n, sweeps = 1024, 100
+    prob = inputs.layered_sinker(n, seed=4)
+    kw = dict(variant="ras", sweeps=sweeps, tile=tile, k=k, overlap=o, seed=1)
+    outs = []
+    for pair in (1, 2, 0):
+        plan = api.stokes_smooth_plan(n, n, api.smooth_params(**kw), dtype, pair_mode=pair)
+        assert plan["path"] == ("stream" if pair == 1 else "tiles")
+        r = Run(api, prob, dtype)
+        r.ctx.set_option(api.STOKES_OPT_PAIRED, pair)
+        r.ctx.profile_reset()
+        r.smooth(**kw)
+        assert r.ctx.profile()["ras"][0] == plan["passes"]
+        outs.append(r.v())
+        r.ctx.close()
+        assert np.array_equal(outs[0][0], outs[-1][0]) and np.array_equal(outs[0][1], outs[-1][1])
