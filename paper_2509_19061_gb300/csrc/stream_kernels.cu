@@ -36,9 +36,14 @@
 // back warp reads the coefficients of its rows there again.  Their only
 // synchronisation is one barrier of the two warps per row.  A cell outside
 // the unknowns has weight zero (its 1/diag is zero), so walls and the outside
-// keep their values within a pass while the fields are finite.  Only unknowns
-// are stored: where a field overflows, the product of zero and infinity next
-// to a wall never reaches the wall's own entry in memory.
+// keep their values while the fields are finite.  Where a field overflows, the
+// product of zero and infinity beside a wall is not zero, and the walls in
+// memory must not take it: row 0 of vy is not stored, and the west wall's entry
+// of vx, which shares a 16-byte store with three unknowns, is the one taken in,
+// kept in shared memory until its row is written (100 sweeps of 8192^2 7.10 ms,
+// 7.06 with computed walls stored; 20 of 4001 x 2999 410 us and 406.  The strip
+// at the wall is on the critical path of its wave: leaving the entry out by
+// smaller stores took 7.46 to 7.72 ms, loading it from memory again 7.97).
 #include <algorithm>
 
 #include "f32x2.cuh"
@@ -55,6 +60,7 @@ constexpr int ST_THREADS = ST_PAIRS * 64;
 constexpr int ST_ROW = ST_FIELDS * ST_COLS;           // elements of a staged row
 constexpr int ST_MIN_SWEEPS = 3, ST_MAX_SWEEPS = 8;   // sweeps of a pass
 constexpr long long ST_MIN_CELLS = 600000;            // smallest grid
+constexpr int ST_WALLS = 16; // rows (a power of two above the rows in flight) whose west wall is kept
 
 // 16-byte asynchronous copy of `bytes` (0 to 16) source bytes, the rest zero
 __device__ __forceinline__ void cp_async16z(uint32_t dst, const float *src, int bytes)
@@ -81,12 +87,29 @@ __device__ __forceinline__ f4 ld4(const float *p)
 {
     return *reinterpret_cast<const f4 *>(p);
 }
-// 16-byte global store of the lanes whose `on` is set, without a branch
-__device__ __forceinline__ void st4_if(float *p, f4 x, bool on)
+// 16-byte global stores of a row of vx and vy by the lanes whose `on` is set,
+// without a branch; vy only if row > 0
+__device__ __forceinline__ void st4_both(float *px, f4 x, float *py, f4 y, bool on, int row)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %3, 0;\n\t@p st.global.v2.b64 [%0], {%1, %2};\n\t}" ::"l"(p),
-                 "l"(x.a.u), "l"(x.b.u), "r"((int)on)
+    asm volatile("{\n\t.reg .pred p, r;\n\tsetp.ne.s32 p, %6, 0;\n\t@p st.global.v2.b64 [%0], {%1, %2};\n\t"
+                 "setp.gt.and.s32 r, %7, 0, p;\n\t@r st.global.v2.b64 [%3], {%4, %5};\n\t}" ::"l"(px),
+                 "l"(x.a.u), "l"(x.b.u), "l"(py), "l"(y.a.u), "l"(y.b.u), "r"((int)on), "r"(row)
                  : "memory");
+}
+// shared store, and load over v, of the lanes whose `on` is set, without a branch
+__device__ __forceinline__ void sts_if(uint32_t p, float v, bool on)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(p), "f"(v),
+                 "r"((int)on)
+                 : "memory");
+}
+__device__ __forceinline__ float lds_if(uint32_t p, float v, bool on)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p ld.shared.f32 %0, [%1];\n\t}"
+                 : "+f"(v)
+                 : "r"(p), "r"((int)on)
+                 : "memory");
+    return v;
 }
 __device__ __forceinline__ f4 operator+(f4 x, f4 y) { return {add2(x.a, y.a), add2(x.b, y.b)}; }
 __device__ __forceinline__ f4 operator-(f4 x, f4 y) { return {sub2(x.a, y.a), sub2(x.b, y.b)}; }
@@ -132,6 +155,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
     using Sh = StreamShape<KL>;
     constexpr int N = Sh::N, D = Sh::D, PF = Sh::PF;
     extern __shared__ __align__(16) float smem[];
+    __shared__ float walls[ST_PAIRS][ST_WALLS]; // vx of column 0 of the last rows taken in, slot = row
     __shared__ StreamEntry held[BATCH ? ST_PAIRS : 1];
     // (the shuffle tells the compiler that the warp number is uniform)
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = (int)threadIdx.x & 31;
@@ -203,12 +227,15 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
         vx[t] = vy[t] = sx[t] = ty[t] = zero;
         if (!SQ) ay[SQ ? 0 : t] = sy[SQ ? 0 : t] = zero;
     }
-    // the unknowns this lane writes: all four columns, or single ones beside the
-    // west wall (vx of column 0) and at the grid's right end
+    // columns this lane writes: all four, or `part` at the grid's right end
     const bool mine = 4 * lane >= a.hl && 4 * lane < a.hl + a.own;
-    const bool full_y = mine && c0 + 4 <= nx, full_x = full_y && c0 > 0;
-    const int part_x = mine && !full_x ? min(nx - c0, 4) : 0, part_y = mine && !full_y ? nx - c0 : 0;
-    const bool edge = __any_sync(0xffffffffu, part_x > 0);
+    const bool full = mine && c0 + 4 <= nx, west = mine && c0 == 0;
+    const int part = mine && !full ? nx - c0 : 0;
+    const bool ragged = __any_sync(0xffffffffu, part > 0);
+    const uint32_t wring = smem_addr(walls[pair]);
+    // (by a branch where that is the faster form: 8192^2 7.11 ms, 7.17 predicated;
+    // the general form 425 us and 410 at 4001 x 2999)
+    constexpr bool BRANCH = SQ && !BATCH;
     int row = jb - n + (back ? KL : 0);       // row the pass completes in this step, as a back warp
     long long q = (long long)row * P + c0;
     int slot = 0;                             // staged slot of the round's first row
@@ -229,6 +256,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
             }
             const float *const in = back ? hand + ((par + u) & 1) * (2 * ST_COLS) : lp + u * ST_ROW;
             f4 ix = ld4(in), iy = ld4(in + ST_COLS);
+            if (BRANCH) {
+                if (!back && west) walls[pair][(jb + rd * N + u) & (ST_WALLS - 1)] = f2lo(ix.a);
+            } else if (!back) {
+                sts_if(wring + ((jb + rd * N + u) & (ST_WALLS - 1)) * 4, f2lo(ix.a), west);
+            }
             auto ld = [&](int f) { return ld4(lp + u * ST_ROW + f * ST_COLS); };
             en[u] = SQ ? mul4(ld(3), cx) : ld(3);
             // the row's coefficients replace those of the row KL steps ago
@@ -273,18 +305,22 @@ __global__ void __launch_bounds__(ST_THREADS, 1)
                 *reinterpret_cast<f4 *>(out) = ix;
                 *reinterpret_cast<f4 *>(out + ST_COLS) = iy;
             } else if (row >= y0 && row < y1) {
-                const bool uy = row > 0; // (row 0 of vy is a wall)
-                st4_if(a.ox + q, ix, full_x);
-                st4_if(a.oy + q, iy, full_y && uy);
-                if (edge) {
-                    float *const px = a.ox + q, *const py = a.oy + q;
-                    if (part_x > 0 && c0 > 0) px[0] = f2lo(ix.a);
-                    if (part_x > 1) px[1] = f2hi(ix.a);
-                    if (part_x > 2) px[2] = f2lo(ix.b);
-                    if (part_x > 3) px[3] = f2hi(ix.b);
-                    if (part_y > 0 && uy) py[0] = f2lo(iy.a);
-                    if (part_y > 1 && uy) py[1] = f2hi(iy.a);
-                    if (part_y > 2 && uy) py[2] = f2lo(iy.b);
+                if (BRANCH) {
+                    if (west) ix.a = pk(walls[pair][row & (ST_WALLS - 1)], f2hi(ix.a));
+                } else {
+                    ix.a = pk(lds_if(wring + (row & (ST_WALLS - 1)) * 4, f2lo(ix.a), west), f2hi(ix.a));
+                }
+                st4_both(a.ox + q, ix, a.oy + q, iy, full, row);
+                if (ragged) {
+                    const bool uy = row > 0;
+                    const f4 o[2] = {ix, iy};
+#pragma unroll
+                    for (int w = 0; w < 2; ++w) {
+                        float *const p = (w ? a.oy : a.ox) + q;
+                        if (part > 0 && (!w || uy)) p[0] = f2lo(o[w].a);
+                        if (part > 1 && (!w || uy)) p[1] = f2hi(o[w].a);
+                        if (part > 2 && (!w || uy)) p[2] = f2lo(o[w].b);
+                    }
                 }
             }
             ++row;
