@@ -30,6 +30,9 @@ constexpr int RB_MAX = 2;     // sweeps of a pass, one warp each
 // fast (20 sweeps 171 us either way); 768^2 takes 253 us by tiles and 232 here,
 // 1024^2 340 and 274, 2000^2 950 and 541.
 constexpr long long RB_MIN_CELLS = 400000;
+// Narrowest grid (a strip sweeps 128 columns however few there are): six sweeps
+// of 32 x 25000 take 103 us by tiles and 142 here, of 48 x 16666 116 and 113.
+constexpr int RB_MIN_NX = 48;
 constexpr int RB_LAG = 4;     // rows from one sweep to the next (three, and one for the hand-over)
 constexpr int RB_D = 12;      // staged rows
 constexpr int RB_PF = RB_D - 1 - RB_LAG * RB_MAX; // rows copied ahead
@@ -261,7 +264,8 @@ int rbgs_stream_passes(int nx, int ny, int sweeps, const RasRun &run)
     // odd pass count costs: 8192^2 one sweep 1014 us, 962 by tiles; two at 640^2
     // 28.4 and 26.4, at 1024^2 37.9 and 39.7.
     const long long least = sweeps == 2 ? 2 * RB_MIN_CELLS : RB_MIN_CELLS;
-    if (!run.allow_tma || run.pair_mode != 1 || sweeps < 2 || (long long)nx * ny < least) return 0;
+    if (!run.allow_tma || run.pair_mode != 1 || sweeps < 2 || nx < RB_MIN_NX || (long long)nx * ny < least)
+        return 0;
     return (sweeps + RB_MAX - 1) / RB_MAX;
 }
 

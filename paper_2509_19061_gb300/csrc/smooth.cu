@@ -19,12 +19,19 @@ bool any_traversal(const SmoothSpec &p)
 // Jacobi in any traversal, and fused Jacobi's sweeps need not each cross the
 // grid before the next begins (20 sweeps of 4001 x 2999: 408 us, 1822 us as 20
 // passes of k_jacobi_rows).  Separate-pass and blocked Jacobi keep their passes.
+// A strip sweeps 128 (FP64: 64) columns however few the grid has, where a tile's
+// window narrows with it: RAS on narrower grids keeps its tiles (24 FP32 sweeps
+// of 12 x 66666 198 us, 219 streamed, of 20 x 40000 351 and 150; eight FP64
+// sweeps of 24 x 33333 673 and 783, of 32 x 25000 918 and 596).  Fused Jacobi
+// streams at any width (FP64, 5 x 60000: 2292 us as passes, 1423).
+constexpr int STREAM_MIN_NX32 = 20, STREAM_MIN_NX64 = 32;
 template <typename T>
 int stream_passes_of(int nx, int ny, const SmoothSpec &p, const RasRun &run)
 {
     if constexpr (sizeof(T) == 4)
         if (p.variant == STOKES_RBGS) return rbgs_stream_passes(nx, ny, p.sweeps, run);
     if (!any_traversal(p)) return 0;
+    if (p.variant == STOKES_RAS && nx < (sizeof(T) == 4 ? STREAM_MIN_NX32 : STREAM_MIN_NX64)) return 0;
     if constexpr (sizeof(T) == 4) return stream_passes((long long)nx * ny, p.sweeps, run);
     else return stream64_passes(nx, ny, p.sweeps, run);
 }

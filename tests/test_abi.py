@@ -160,3 +160,20 @@ def test_smooth_plan_without_device(lib):
                                                    ctypes.byref(api.stokes_smooth_plan_info()))
                 raise api.StokesError(st, "dtype")
             plan(64, **kw)
+
+
+def test_narrow_grids_keep_their_tiles(lib):
+    """A row-streaming strip sweeps its full width however few columns the grid
+    has: RAS and RBGS on narrow grids run on tiles, fused Jacobi streams."""
+    from paper_2509_19061_gb300 import api
+
+    def path(nx, ny, dtype, **kw):
+        return api.stokes_smooth_plan(nx, ny, api.smooth_params(**kw), dtype, max_cluster=16)["path"]
+
+    exact = dict(variant="ras", sweeps=8, tile=(32, 32), k=4, overlap=3)
+    for dtype, nx in (("f32", 20), ("f64", 32)):
+        assert path(nx - 1, 200000, dtype, **exact) == "tiles" and path(nx, 200000, dtype, **exact) == "stream"
+        assert path(3, 250000, dtype, variant="fused", sweeps=8) == "stream"
+        assert path(250000, 3, dtype, **exact) == "stream"
+    assert path(47, 200000, "f32", variant="rbgs", sweeps=6) == "passes"
+    assert path(48, 200000, "f32", variant="rbgs", sweeps=6) == "stream"

@@ -869,12 +869,13 @@ def test_row_streaming_keeps_the_walls_of_an_overflowing_field(api, nx, ny, squa
 
 
 @pytest.mark.parametrize("nx,ny,sweeps,square", [
-    (1121, 400, 3, True), (1120, 801, 2, False), (4, 210000, 2, False), (210000, 4, 2, True), (960, 450, 5, False),
+    (1121, 400, 3, True), (1120, 801, 2, False), (48, 16700, 2, False), (210000, 4, 2, True), (960, 450, 5, False),
 ])
 def test_rbgs_streams_two_sweeps_a_pass(api, nx, ny, sweeps, square):
     """Sizes and sweep counts at which red-black Gauss-Seidel does stream (the
     launch counts say so): one pass of two sweeps with its copy back, an odd last
-    sweep, grids of four columns and rows; value for value the tile kernel's."""
+    sweep, the narrowest grid and one of four rows; value for value the tile
+    kernel's."""
     prob = rand_problem(nx, ny, 98, lx=1.0, ly=ny / nx if square else 0.7)
     vx, vy = inputs.random_velocity(nx, ny, 99, 0.1)
     vx[:, 0], vx[:, nx], vy[0], vy[ny] = 0.3, -0.2, 0.1, 0.4
