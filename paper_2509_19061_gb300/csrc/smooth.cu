@@ -46,6 +46,10 @@ int stream_passes_of(int nx, int ny, const SmoothSpec &p, const RasRun &run)
 // tiles with k = 4 6.5 for four), so the window height with the least product is
 // taken.  With the middle levels' tiles as given: 512^2 Uzawa (32 x 32, k = 4)
 // 25.0 ms, now 24.1; 8 CG cycles of 1024^2 (48 x 32, k = 8) 7.28 and 7.11.
+// Given tiles that run the sweeps in one pass of one wave stay where their
+// windows are narrower still, up to 48 columns (one a thread), and the sweeps
+// at most four (four sweeps of 200^2 on 32 x 32 tiles 14.4 us, 16.5 on chosen
+// ones; at 500^2, two waves, 18.5 and 16.5).
 constexpr long long FREE_MAX_CELLS = 600000; // where the row streaming starts
 template <typename T>
 SmoothSpec tiles_of(int nx, int ny, const SmoothSpec &p, const RasRun &run)
@@ -53,6 +57,8 @@ SmoothSpec tiles_of(int nx, int ny, const SmoothSpec &p, const RasRun &run)
     if (sizeof(T) != 4 || p.variant != STOKES_RAS || p.sweeps < 1 || !any_traversal(p) || !run.allow_tma ||
         run.pair_mode != 1 || p.k > 8 || nx < 64 || ny < 40 || (long long)nx * ny >= FREE_MAX_CELLS)
         return p;
+    const long long given = (long long)((nx + p.ti - 1) / p.ti + 1) * ((ny + p.tj - 1) / p.tj + 1); // (shifted)
+    if (p.sweeps <= p.k && p.sweeps <= 4 && given <= 152 && p.ti + 2 * p.overlap + 2 <= 48) return p;
     SmoothSpec q = p;
     const int passes = (p.sweeps + 7) / 8;
     q.k = (p.sweeps + passes - 1) / passes;

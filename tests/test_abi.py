@@ -177,3 +177,18 @@ def test_narrow_grids_keep_their_tiles(lib):
         assert path(250000, 3, dtype, **exact) == "stream"
     assert path(47, 200000, "f32", variant="rbgs", sweeps=6) == "passes"
     assert path(48, 200000, "f32", variant="rbgs", sweeps=6) == "stream"
+
+
+def test_one_wave_of_given_tiles_stays(lib):
+    """Middle FP32 grids whose given tiles run the sweeps in one pass of one wave
+    keep them; more sweeps, more tiles or wider windows take chosen ones."""
+    from paper_2509_19061_gb300 import api
+
+    def tile(n, sweeps, tile=(32, 32), k=4, overlap=3):
+        plan = api.stokes_smooth_plan(n, n, api.smooth_params("ras", sweeps, tile, k, overlap), "f32", max_cluster=16)
+        assert plan["path"] == "tiles"
+        return plan["tile"]
+
+    assert tile(200, 4) == tile(330, 3) == (32, 32)
+    for other in (tile(200, 5), tile(400, 4), tile(200, 4, (56, 32)), tile(200, 8, (30, 30), 8, 7)):
+        assert other not in ((32, 32), (30, 30))
