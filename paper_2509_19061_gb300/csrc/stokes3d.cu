@@ -1044,7 +1044,12 @@ int smooth_impl(stokes3d_ctx *c, T *vx, T *vy, T *vz, const T *p, const stokes3d
     // with k = 2; 192^3 1777, 2160 to 3529; 320^3 6880, 9209 to 16796.  FP64: 47^3
     // 498, 683 to 2544; 192^3 17.7 ms, 30 to 107.  (k = 1 keeps its tiles: 1823 us
     // at 192^3 in FP32, but 12.4 ms for two sweeps of 320^3 in FP64, 13.3 fused.)
-    const bool exact = prm->variant == STOKES_RAS && prm->k >= 2 && prm->overlap >= prm->k - 1 &&
+    // A pass's rows are whole warps of columns, a tile as wide as it is given, so
+    // narrow boxes keep their tiles: four FP32 sweeps of 40 x 400 x 150 on 8^3
+    // tiles with k = 2 452 us, 517 fused, of 64 x 200 x 200 457 and 385; FP64 12 x
+    // 450 x 450 4256 and 5963, 24 x 300 x 300 3478 and 2677.
+    const bool wide = c->nx >= (sizeof(T) == 4 ? 64 : 20);
+    const bool exact = prm->variant == STOKES_RAS && prm->k >= 2 && prm->overlap >= prm->k - 1 && wide &&
                        (long long)c->nx * c->ny * c->nz >= (sizeof(T) == 4 ? 2000000 : 100000);
     if (exact && prm->shift_mode == STOKES_SHIFT_LIST)
         for (int t = 0; t < (prm->sweeps + prm->k - 1) / prm->k; ++t)

@@ -366,3 +366,24 @@ def test_3d_errors(api):
     assert e.value.status == api.STOKES_ERR_ARG
     torch.cuda.synchronize()
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,n,fused", [("f32", (40, 240, 215), False), ("f32", (64, 180, 180), True),
+                                           ("f64", (12, 120, 80), False), ("f64", (20, 90, 70), True)])
+def test_narrow_boxes_keep_their_tiles(api, dtype, n, fused):
+    """An exact RAS schedule (overlap >= k - 1) on a large box runs as fused Jacobi
+    where its rows fill the warps, a launch a sweep, and on its tiles where they do
+    not, a launch an outer iteration; the same values."""
+    prob = problem(*n, 21)
+    v0 = inputs.random_velocity3d(*n, 22, 0.1)
+    r = Run3(api, prob, dtype, v0)
+    before = r.ctx.kernels()
+    r.smooth(variant="ras", sweeps=8, tile=(8, 8, 8), k=2, overlap=1, seed=3)
+    ras = r.ctx.kernels() - before
+    s = Run3(api, prob, dtype, v0)
+    before = s.ctx.kernels()
+    s.smooth(variant="fused", sweeps=8)
+    jacobi = s.ctx.kernels() - before
+    assert ras == (jacobi if fused else jacobi - 4)
+    for x, y in zip(r.get(), s.get()):
+        assert np.array_equal(x, y)
