@@ -437,12 +437,16 @@ cudaError_t mg_residual_restrict(const MgLevel &f, const MgLevel &c, cudaStream_
         return op_rows_restrict(make_grid<T>(f.nx, f.ny, f.pitch, f.hx, f.hy), (const T *)f.ec, (const T *)f.en,
                                 (const T *)f.bx, (const T *)f.by, (const T *)f.vx, (const T *)f.vy, (T *)c.bx,
                                 (T *)c.by, c.pitch, s);
-    const cudaError_t e = mg_residual<T>(f, s);
-    if (e != cudaSuccess) return e;
-    k_restrict<T><<<grid2d(c.nx + 1, c.ny + 1), dim3(BX, BY), 0, s>>>(f.nx, f.ny, f.pitch, c.nx, c.ny, c.pitch,
-                                                                       (const T *)f.rx, (const T *)f.ry, (T *)c.bx,
-                                                                       (T *)c.by);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        const cudaError_t e = mg_residual<T>(f, s);
+        if (e != cudaSuccess) return e;
+        k_restrict<T><<<grid2d(c.nx + 1, c.ny + 1), dim3(BX, BY), 0, s>>>(f.nx, f.ny, f.pitch, c.nx, c.ny, c.pitch,
+                                                                           (const T *)f.rx, (const T *)f.ry, (T *)c.bx,
+                                                                           (T *)c.by);
+        return cudaGetLastError();
+    } else {
+        return cudaErrorInvalidValue; // (FP32 levels always take the fused form)
+    }
 }
 
 template <typename T>

@@ -71,17 +71,6 @@ __device__ __forceinline__ void stq(float *p, const Q4 &v)
 __device__ __forceinline__ float west(const Q4 &v) { return __shfl_up_sync(0xffffffffu, v.e[3], 1); }
 __device__ __forceinline__ float east(const Q4 &v) { return __shfl_down_sync(0xffffffffu, v.e[0], 1); }
 
-__device__ __forceinline__ void cp_async16z(uint32_t dst, const float *src, int bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // vx of the columns K, K + 2 of row j from its neighbours (gs_half's
 // operations): rows j + 1 and j - 1 of vx, rows j + 1 and j of vy
 template <int K, bool SQ>

@@ -70,17 +70,6 @@ __device__ __forceinline__ D2 diff_east(D2 x)
     return {r_sub(x.b, x.a), r_sub(__shfl_down_sync(0xffffffffu, x.a, 1), x.b)};
 }
 
-__device__ __forceinline__ void cp_async16z(uint32_t dst, const double *src, int bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // blockDim.x / 32 sweeps of strip blockIdx.x % strips, segment blockIdx.x / strips
 template <bool SQ>
 __global__ void __launch_bounds__(S8_MAX * 32, 4) k_stream64(const __grid_constant__ Stream64 a)

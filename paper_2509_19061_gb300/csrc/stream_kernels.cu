@@ -62,17 +62,6 @@ constexpr int ST_MIN_SWEEPS = 3, ST_MAX_SWEEPS = 8;   // sweeps of a pass
 constexpr long long ST_MIN_CELLS = 600000;            // smallest grid
 constexpr int ST_WALLS = 16; // rows (a power of two above the rows in flight) whose west wall is kept
 
-// 16-byte asynchronous copy of `bytes` (0 to 16) source bytes, the rest zero
-__device__ __forceinline__ void cp_async16z(uint32_t dst, const float *src, int bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 // barrier of the two warps of a pair
 __device__ __forceinline__ void pair_sync(int pair)
 {

@@ -1,6 +1,6 @@
 // tma.h -- tensor-memory-accelerator helpers (internal): host-side tensor map
-// encoding through the driver entry point, device-side mbarrier and 2D bulk
-// tensor copies written as inline PTX for sm_103a.
+// encoding through the driver entry point, device-side mbarrier, 2D bulk
+// tensor copies and 16-byte asynchronous copies written as inline PTX for sm_103a.
 #pragma once
 
 #include <cuda.h>
@@ -76,6 +76,20 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
                  " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_addr(dst)),
                  "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
                  : "memory");
+}
+
+// 16-byte asynchronous copy of `bytes` (0 to 16) source bytes, the rest zero, in
+// groups: wait until at most N of this thread's groups are in flight
+template <typename T>
+__device__ __forceinline__ void cp_async16z(uint32_t dst, const T *src, int bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 #endif
 
