@@ -71,7 +71,7 @@ int alloc_level(MgLevel &l, int nx, int ny, double hx, double hy, size_t es, boo
         if (f >= 6 && !(f < 8 ? resid : inv)) continue;
         cudaError_t e = cudaMalloc(fs[f], l.elems * es);
         if (e == cudaSuccess) e = cudaMemsetAsync(*fs[f], 0, l.elems * es, s);
-        if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? STOKES_ERR_OOM : STOKES_ERR_CUDA;
+        if (e != cudaSuccess) return cuda_fail(e, "a multigrid level");
     }
     return STOKES_OK;
 }
@@ -99,7 +99,8 @@ int n_unknowns(int nx, int ny) { return ny * (nx - 1) + (ny - 1) * nx; }
 
 #define CKS(expr)                                                                                                  \
     do {                                                                                                           \
-        if ((expr) != cudaSuccess) return STOKES_ERR_CUDA;                                                         \
+        const cudaError_t e_ = (expr);                                                                             \
+        if (e_ != cudaSuccess) return cuda_fail(e_, #expr);                                                        \
     } while (0)
 
 template <typename Ti>
@@ -136,7 +137,7 @@ int build(MgHierarchy *h, const MgOuter &o, int levels, int coarsest, cudaStream
     for (int l = 0; l < L; ++l) h->vel_bytes += 2 * field_bytes(l);
     {
         const cudaError_t e = cudaMalloc(&h->vel, h->vel_bytes);
-        if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? STOKES_ERR_OOM : STOKES_ERR_CUDA;
+        if (e != cudaSuccess) return cuda_fail(e, "the levels' velocities");
         CKS(cudaMemsetAsync(h->vel, 0, h->vel_bytes, s));
         unsigned char *at = (unsigned char *)h->vel;
         for (int l = 0; l < L; ++l) {
@@ -165,9 +166,10 @@ int build(MgHierarchy *h, const MgOuter &o, int levels, int coarsest, cudaStream
     const MgLevel &lc = h->lv[L - 1];
     h->n = n_unknowns(lc.nx, lc.ny);
     const size_t nn = (size_t)h->n * h->n;
-    if (cudaMalloc(&h->A, nn * 8) != cudaSuccess || cudaMalloc(&h->W, nn * 8) != cudaSuccess ||
-        cudaMalloc(&h->Ainv, nn * 8) != cudaSuccess || cudaMalloc(&h->dstatus, sizeof(int)) != cudaSuccess)
-        return STOKES_ERR_OOM;
+    CKS(cudaMalloc(&h->A, nn * 8));
+    CKS(cudaMalloc(&h->W, nn * 8));
+    CKS(cudaMalloc(&h->Ainv, nn * 8));
+    CKS(cudaMalloc(&h->dstatus, sizeof(int)));
     CKS(cudaMemsetAsync(h->dstatus, 0, sizeof(int), s));
     CKS(mg_dense_setup<Ti>(lc, h->n, h->A, h->W, h->Ainv, h->dstatus, s));
     int bad = 0;

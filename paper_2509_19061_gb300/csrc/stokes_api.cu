@@ -23,6 +23,7 @@ thread_local char g_cuda_err[256] = "";
 int stokes::cuda_fail(cudaError_t e, const char *where)
 {
     std::snprintf(g_cuda_err, sizeof g_cuda_err, "%s: %s", where, cudaGetErrorString(e));
+    cudaGetLastError(); // reported here: the next launch must not find it again
     return e == cudaErrorMemoryAllocation ? STOKES_ERR_OOM : STOKES_ERR_CUDA;
 }
 
@@ -293,7 +294,6 @@ int smooth_impl(stokes_ctx *c, T *vx, T *vy, const stokes_smooth_params *p, int 
                 cudaFree(c->sy2);
                 c->sx2 = c->sy2 = nullptr;
                 if (!optional || st != STOKES_ERR_OOM) return st;
-                cudaGetLastError();
             }
         }
     }
@@ -360,17 +360,38 @@ MgOuter outer_of(const stokes_ctx *c)
     return o;
 }
 
-// work vectors of the outer solve, allocated on first use
-// The flux coefficients of the current viscosity (allocated on first use).
+// What a call needs beyond the context is allocated on first use, each buffer
+// where it is missing: an allocation that fails halfway leaves the rest missing,
+// and the next call goes on from there.
+int ensure_field(stokes_ctx *c, void **p) { return *p ? STOKES_OK : alloc_field(c, p); }
+
+template <typename P>
+int ensure_device(P **p, size_t bytes)
+{
+    if (!*p) CK(cudaMalloc(p, bytes));
+    return STOKES_OK;
+}
+
+template <typename P>
+int ensure_pinned(P **p, size_t bytes)
+{
+    if (!*p) CK(cudaMallocHost(p, bytes));
+    return STOKES_OK;
+}
+
+#define ENSURE(call)                                                                                               \
+    do {                                                                                                           \
+        const int st_ = (call);                                                                                    \
+        if (st_ != STOKES_OK) return st_;                                                                          \
+    } while (0)
+
+// the flux coefficients of the current viscosity
 template <typename T>
 int ensure_coef(stokes_ctx *c, const KrylovView &kv)
 {
-    if (!c->cax) {
-        int st = alloc_field(c, &c->cax);
-        if (st == STOKES_OK) st = alloc_field(c, &c->cay);
-        if (st != STOKES_OK) return st;
-        c->coef_version = -1;
-    }
+    if (!c->cax || !c->cay) c->coef_version = -1;
+    ENSURE(ensure_field(c, &c->cax));
+    ENSURE(ensure_field(c, &c->cay));
     if (c->coef_version != c->eta_version) {
         RUN(STOKES_K_COPY, 1, kry_coef<T>(kv, grid_of<T>(c), (const T *)c->eta_c, (T *)c->cax, (T *)c->cay, c->stream));
         c->coef_version = c->eta_version;
@@ -378,23 +399,20 @@ int ensure_coef(stokes_ctx *c, const KrylovView &kv)
     return STOKES_OK;
 }
 
+// work vectors of the outer solve
 int ensure_work(stokes_ctx *c)
 {
-    if (c->kw[0]) return STOKES_OK;
-    for (void *&w : c->kw) {
-        const int st = alloc_field(c, &w);
-        if (st != STOKES_OK) return st;
-    }
-    CK(cudaMalloc(&c->kpartials, (size_t)krylov_partials() * 2 * sizeof(double)));
-    CK(cudaMalloc(&c->kout, 6 * sizeof(double))); // three pairs of reduction results
-    CK(cudaMallocHost(&c->hout, 2 * sizeof(double)));
-    return STOKES_OK;
+    for (void *&w : c->kw) ENSURE(ensure_field(c, &w));
+    ENSURE(ensure_device(&c->kpartials, (size_t)krylov_partials() * 2 * sizeof(double)));
+    ENSURE(ensure_device(&c->kout, 6 * sizeof(double))); // three pairs of reduction results
+    return ensure_pinned(&c->hout, 2 * sizeof(double));
 }
 
 // Inner-precision work vectors of the refinement mode (krylov = 2).
 int ensure_inner_work(stokes_ctx *c, int dtype)
 {
-    if (c->iw[0] && c->iw_dtype == dtype) return STOKES_OK;
+    if (c->iw_dtype == dtype) return STOKES_OK;
+    c->iw_dtype = -1; // (until all are there)
     for (void *&w : c->iw)
         if (w) {
             cudaFree(w);
@@ -694,20 +712,15 @@ int uzawa_impl(stokes_ctx *c, T *vx, T *vy, T *p, const stokes_uzawa_params *u, 
                double *final_e)
 {
     const GridDesc<T> g = grid_of<T>(c);
-    if (!c->uz_partials) {
-        CK(cudaMalloc(&c->uz_partials, (size_t)uzawa_partials() * sizeof(double)));
-        CK(cudaMalloc(&c->uz_scal, 2 * sizeof(double)));
-    }
+    ENSURE(ensure_device(&c->uz_partials, (size_t)uzawa_partials() * sizeof(double)));
+    ENSURE(ensure_device(&c->uz_scal, 2 * sizeof(double)));
     if (u->lithostatic_init)
         RUN(STOKES_K_RHS, 4,
             uz_lithostatic<T>(g, c->hy, (const T *)c->fy, p, c->uz_partials, c->uz_scal + 1, c->stream));
     const bool cont = u->theta_interval > 0 && u->theta_stages > 1;
     if (cont) {
-        if (!c->eta_c0) {
-            int st = alloc_field(c, &c->eta_c0);
-            if (st == STOKES_OK) st = alloc_field(c, &c->eta_n0);
-            if (st != STOKES_OK) return st;
-        }
+        ENSURE(ensure_field(c, &c->eta_c0));
+        ENSURE(ensure_field(c, &c->eta_n0));
         CK(cudaMemcpyAsync(c->eta_c0, c->eta_c, c->elems * c->esize, cudaMemcpyDeviceToDevice, c->stream));
         CK(cudaMemcpyAsync(c->eta_n0, c->eta_n, c->elems * c->esize, cudaMemcpyDeviceToDevice, c->stream));
         RUN(STOKES_K_COPY, 2,
@@ -718,18 +731,16 @@ int uzawa_impl(stokes_ctx *c, T *vx, T *vy, T *p, const stokes_uzawa_params *u, 
     // Anderson acceleration (Algorithm 1): history of F(x_i) and r_i = F(x_i) - x_i
     const int depth = u->anderson_depth, slots = depth + 1;
     const size_t fbytes = c->elems * c->esize;
-    if (depth > 0 && (int)c->aa.size() < 6 * slots + 3) {
+    if (depth > 0) {
         while ((int)c->aa.size() < 6 * slots + 3) {
             void *f = nullptr;
             const int st0 = alloc_field(c, &f);
+            if (f) c->aa.push_back(f);
             if (st0 != STOKES_OK) return st0;
-            c->aa.push_back(f);
         }
-        if (!c->aa_partials) {
-            CK(cudaMalloc(&c->aa_partials, (size_t)uzawa_partials() * AA_MAX * sizeof(double)));
-            CK(cudaMalloc(&c->aa_out, AA_MAX * sizeof(double)));
-            CK(cudaMallocHost(&c->aa_hout, AA_MAX * sizeof(double)));
-        }
+        ENSURE(ensure_device(&c->aa_partials, (size_t)uzawa_partials() * AA_MAX * sizeof(double)));
+        ENSURE(ensure_device(&c->aa_out, AA_MAX * sizeof(double)));
+        ENSURE(ensure_pinned(&c->aa_hout, AA_MAX * sizeof(double)));
     }
     auto fld = [&](int slot, int kind, int comp) { return (T *)c->aa[(size_t)(slot * 6 + kind * 3 + comp)]; };
     T *const xo[3] = {depth > 0 ? (T *)c->aa[6 * slots] : nullptr, depth > 0 ? (T *)c->aa[6 * slots + 1] : nullptr,
