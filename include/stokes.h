@@ -206,7 +206,8 @@ int stokes_apply_operator(stokes_ctx *ctx, const void *vx, const void *vy, const
  * RBGS one per sweep.  Where the result is the same value for value, fewer run:
  * RAS with o >= k - 1 (any shifts) and fused Jacobi up to eight sweeps a pass on
  * large grids and all sweeps in one launch, in place, on small ones; RBGS in FP32
- * two sweeps a pass on large grids. */
+ * two sweeps a pass on large grids (RAS and RBGS not on narrow ones;
+ * stokes_smooth_plan says what a call runs). */
 int stokes_smooth(stokes_ctx *ctx, void *vx, void *vy, const void *p, const stokes_smooth_params *params);
 
 /* Energy residual sums of Sec. 6.4, accumulated in FP64:

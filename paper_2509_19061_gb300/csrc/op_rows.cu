@@ -23,7 +23,8 @@
 // 4096^2: 149 us, 328 as a residual and a restriction a level.
 //
 // Operations and their order are those of stencil.cuh, so M v has the bits of
-// the other kernels.
+// the other kernels.  G p is subtracted by one fused multiply-add, where k_apply
+// rounds the product first: M v + G p may differ from it in the last bit.
 #include <algorithm>
 
 #include "batch.h"

@@ -22,11 +22,11 @@
 // registers, which pays for four columns per lane: two independent chains of
 // arithmetic, half the shuffles and half the spare columns of a two-column
 // form with all sweeps in one warp (648 us a pass of 7.7 sweeps at 8192^2,
-// against 465 here and 915 for the pair kernel's 48 x 64 tiles).
+// against 470 here and 915 for the pair kernel's 48 x 64 tiles).
 //
 // Bounds (8192^2, 100 sweeps in 13 passes): 40 bytes a cell and pass (eight
 // fields read, two written) take 400 us at the measured copy rate, the packed
-// arithmetic about 360 us of the FMA pipe; 465 us is 0.86 of that copy rate.
+// arithmetic about 360 us of the FMA pipe; 470 us is 0.85 of that copy rate.
 // On the way: the rows' loads and copies at the end of a step instead of its
 // start 564 us; register copies left by a ring of KL slots under state that
 // rotates through KL + 1 another 100 us.
@@ -367,7 +367,10 @@ int stream_passes(long long cells, int sweeps, const RasRun &run)
     if (!run.allow_tma || run.pair_mode != 1 || sweeps < ST_MIN_SWEEPS) return 0;
     // Below this a segment's 2 n extra rows outweigh the tiles' halo: 40 sweeps
     // take 101 us either way at 768^2, 80 (48 x 64 tiles: 70) at 512^2 and 111
-    // (132) at 1024^2.
+    // (132) at 1024^2.  In a batch the instances' strips fill the wave together,
+    // half-empty ones too (20 sweeps, against 48 x 64 tiles: 200 grids of 64^2 101
+    // us and 180, 3000 of 32^2 551 and 892, 4000 of 16^2 474 and 595; three sweeps
+    // of 200 of 64^2 46 and 61).
     if (cells < ST_MIN_CELLS) return 0;
     return (sweeps + ST_MAX_SWEEPS - 1) / ST_MAX_SWEEPS;
 }
